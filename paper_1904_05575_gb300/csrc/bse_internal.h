@@ -142,12 +142,32 @@ void davidson_fp64(int n, const bse_c128* A, const bse_c128* B, int64_t ld, int 
 
 // Hermitian matrix-vector blocks on the tensor cores (build_mixed.cu): A and
 // B split once; apply writes AV = A V and BV = B V (n x k, column-major, ld n).
+// Nothing here waits for the device except tc_matvec_check, which throws
+// BSE_ERR_TIMEOUT if a bounded wait expired in a product since the last check.
 struct TcMatvec;
 TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t ld, int precision,
                            int kmax, cudaStream_t stream);
 void tc_matvec_apply(TcMatvec* m, const bse_c128* V, int k, bse_c128* AV, bse_c128* BV,
                      cudaStream_t stream);
+void tc_matvec_check(TcMatvec* m, cudaStream_t stream);
 void tc_matvec_destroy(TcMatvec* m);
+
+// One vector's product with A in two halves, for a caller that forms the
+// vector and uses the result in its own kernels: the caller writes the
+// vector's pieces to row 0 of the 3P planes vplanes (-Im, Re, Im of each
+// piece, vplane elements apart), tc_matvec_products leaves the K segments'
+// partial sums in part [nseg][n] (to be added in that order in FP32), and
+// diag is A's diagonal (element i at i (diag_ld + 1)), not part of the sums.
+struct TcMatvecIo {
+  void* vplanes;
+  int64_t vplane;
+  int pieces, nseg;
+  const float2* part;
+  const double2* diag;
+  int64_t diag_ld;
+};
+TcMatvecIo tc_matvec_io(const TcMatvec* m);
+void tc_matvec_products(TcMatvec* m, cudaStream_t stream);
 
 // Batched plans (build_mixed.cu).
 struct BatchPlan;

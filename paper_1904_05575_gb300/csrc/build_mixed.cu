@@ -1064,10 +1064,14 @@ int num_sms() {
   return n;
 }
 
-// d_err: two ints, the error bits and the counter of the dynamic unit hand-out
+// d_err: two ints, the error bits and the counter of the dynamic unit hand-out.
+// static_order: units in the fixed order b, b + grid, ... (no counter, no
+// memset node): for launches whose units share no operand that would have to
+// stay in L2.
 template <class Epi>
 void launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const tc::Tile* d_tiles, int ntiles,
-                 const tc::GemmShape& sh, const Epi& epi, int* d_err, cudaStream_t s) {
+                 const tc::GemmShape& sh, const Epi& epi, int* d_err, cudaStream_t s,
+                 bool static_order = false) {
   if (ntiles == 0) return;
   const size_t smem = tc::gemm_smem_bytes(sh);
   const bool seg = sh.ksegs > 1;
@@ -1096,7 +1100,7 @@ void launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const tc::Tile* d
   const int units = (ntiles + sh.group - 1) / sh.group;
   const int grid = std::min<int>(units, num_sms());
   int* units_taken = nullptr;
-  if (units > grid) {   // more than one round of units: hand them out in order of need
+  if (units > grid && !static_order) {   // more than one round of units: hand them out in order of need
     units_taken = d_err + 1;
     BSE_CUDA(cudaMemsetAsync(units_taken, 0, sizeof(int), s));
   }
@@ -2176,6 +2180,7 @@ namespace {
 struct MatvecEpi {
   double2* out;
   int64_t ld;
+  int ncols;                       // columns of the block
   const double2* diag = nullptr;   // the matrix (its diagonal is added in FP64), or NULL
   int64_t diag_ld = 0;
   const double2* v = nullptr;      // the FP64 block V, column-major with leading dimension ld
@@ -2186,7 +2191,7 @@ struct MatvecEpi {
     if (diag) d = diag[r * (diag_ld + 1)];
 #pragma unroll
     for (int j = 0; j < 32; ++j)
-      if (c0 + j < t.n_valid) {
+      if (t.n0 + c0 + j < ncols) {
         const int64_t o = r + (int64_t)(t.n0 + c0 + j) * ld;
         double2 y = make_double2(f32_to_f64_bits(re[j]), f32_to_f64_bits(im[j]));
         if (diag) {
@@ -2198,17 +2203,90 @@ struct MatvecEpi {
       }
   }
 };
+
+// One K segment's sums of a tile (Tile::prob = segment), [segment][column][row].
+struct MatvecPartEpi {
+  float2* part;
+  int64_t n;
+  int ncols;
+  __device__ __forceinline__ void operator()(const tc::Tile& t, int row, int c0, const float* re,
+                                             const float* im) const {
+    float2* dst = part + ((int64_t)t.prob * ncols + t.n0 + c0) * n + t.out_row0 + row;
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (t.n0 + c0 + j < ncols) dst[(int64_t)j * n] = make_float2(re[j], im[j]);
+  }
+};
+
+// out[:, c] = the segments' sums added in segment order (FP32, the order of
+// the segmented tiles' own epilogue: the same bits) + diag * v
+__global__ void __launch_bounds__(256) k_matvec_reduce(int n, int ncols, int nseg,
+                                                       const float2* __restrict__ part,
+                                                       const double2* diag, int64_t diag_ld,
+                                                       const double2* v, double2* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
+  if (i >= n) return;
+  float re = 0.f, im = 0.f;
+  const float2* p = part + (int64_t)c * n + i;
+  const int64_t step = (int64_t)ncols * n;
+#pragma unroll 8
+  for (int sgm = 0; sgm < nseg; ++sgm) {
+    const float2 t = p[sgm * step];
+    re += t.x;
+    im += t.y;
+  }
+  double2 y = make_double2(f32_to_f64_bits(re), f32_to_f64_bits(im));
+  const int64_t o = i + (int64_t)c * n;
+  if (diag) {
+    const double2 d = diag[i * (diag_ld + 1)], x = v[o];
+    y.x += d.x * x.x - d.y * x.y;
+    y.y += d.x * x.y + d.y * x.x;
+  }
+  out[o] = y;
+}
+
+constexpr size_t kMatvecPartBytes = (size_t)512 << 20;   // most scratch for split-K partial sums
 }  // namespace
 
+// A block's products run in one of two forms with the same bits.  Split K:
+// one tile per 128 rows and K segment, partial sums added by k_matvec_reduce;
+// a row tile alone would keep only n / 128 of the SMs busy, each streaming
+// its rows at one SM's share of the bandwidth (N = 4,860: 38 blocks, 200 us per
+// product; split over 38 segments: bound by reading the planes).  Whole K per
+// tile where the partial sums would exceed kMatvecPartBytes (wide blocks of
+// large matrices: enough tiles by themselves).
 struct TcMatvec {
-  int n = 0, Kp = 0, pieces = 3, planes = 6, kmax = 0, kmax_rows = 0, nt = 0, max_tiles = 0;
+  int n = 0, Kp = 0, pieces = 3, planes = 6, kmax = 0, kmax_rows = 0, nt = 0;
+  int seg_len = 0, nseg = 0;     // K steps per segment, segments
+  int split_cols = 0;            // widest block of the split-K form
   bool has_b = false;
   const bse_c128* A = nullptr;   // caller's A (its diagonal, in FP64)
   int64_t ld = 0;
-  DevMem ap, bp, vp, tiles, err;
+  std::unique_ptr<DeviceBuffer> ap, bp, vp, part, err;
+  struct TileList {
+    std::vector<tc::Tile> host;            // kept until the copy has been read
+    std::unique_ptr<DeviceBuffer> dev;
+  };
+  std::map<int, TileList> split_tiles, whole_tiles;   // by number of column tiles
   CUtensorMap ma_a{}, ma_b{}, mb_v{};
-  tc::GemmShape sh{};
+  tc::GemmShape sh{}, sh_seg{};
 };
+
+namespace {
+const TcMatvec::TileList& matvec_tiles(TcMatvec* m, int ncol, bool split, cudaStream_t s) {
+  TcMatvec::TileList& tl = (split ? m->split_tiles : m->whole_tiles)[ncol];
+  if (tl.dev) return tl;
+  for (int m0 = 0; m0 < m->n; m0 += tc::BM)
+    for (int sg = 0; sg < (split ? m->nseg : 1); ++sg)
+      for (int c = 0; c < ncol; ++c)
+        tl.host.push_back({m0, std::min(tc::BM, m->n - m0), c * m->nt, c * m->nt, m->nt, m0, sg,
+                           sg * m->seg_len});
+  tl.dev.reset(new DeviceBuffer(tl.host.size() * sizeof(tc::Tile), s));
+  BSE_CUDA(cudaMemcpyAsync(tl.dev->ptr, tl.host.data(), tl.host.size() * sizeof(tc::Tile),
+                           cudaMemcpyHostToDevice, s));
+  return tl;
+}
+}  // namespace
 
 TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t ld, int precision,
                            int kmax, cudaStream_t s) {
@@ -2218,61 +2296,100 @@ TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t 
   m->planes = 2 * m->pieces;
   m->Kp = round_up(n, tc::BK);
   m->kmax = kmax;
-  m->kmax_rows = round_up(kmax, 32);
-  m->nt = tile_cols(m->kmax_rows, m->Kp);
+  // a single vector: tiles of 8 columns, split K always (its partial sums are
+  // the smallest); the planes of one tile take 27 instead of 34 KB per K step
+  const bool single = kmax == 1;
+  m->kmax_rows = single ? 8 : round_up(kmax, 32);
+  m->nt = single ? 8 : tile_cols(m->kmax_rows, m->Kp);
   m->sh = make_shape(m->nt, m->Kp, m->pieces);
+  // the segments of the whole-K form (see mma_role); the last one may run past
+  // the padded K, where the planes read as zero
+  m->seg_len = (m->sh.kchunks + m->sh.ksegs - 1) / m->sh.ksegs;
+  m->nseg = (m->sh.kchunks + m->seg_len - 1) / m->seg_len;
+  m->sh_seg = m->sh;
+  m->sh_seg.kchunks = m->seg_len;
+  m->sh_seg.ksegs = 1;
   m->has_b = B != nullptr;
   m->A = A;
   m->ld = ld;
-  m->max_tiles = ((n + tc::BM - 1) / tc::BM) * ((kmax + m->nt - 1) / m->nt);
+  const size_t col_bytes = (size_t)m->nseg * n * sizeof(float2);
+  m->split_cols = (int)std::max<size_t>(1, std::min<size_t>(kmax, kMatvecPartBytes / col_bytes));
+  m->part.reset(new DeviceBuffer(m->split_cols * col_bytes, s));
   const size_t mat_bytes = (size_t)m->planes * n * m->Kp * 2;
-  m->ap = DevMem(mat_bytes);
-  if (B) m->bp = DevMem(mat_bytes);
+  m->ap.reset(new DeviceBuffer(mat_bytes, s));
+  if (B) m->bp.reset(new DeviceBuffer(mat_bytes, s));
   const size_t v_bytes = (size_t)tc::b_planes(m->pieces) * m->kmax_rows * m->Kp * 2;
-  m->vp = DevMem(v_bytes);
-  BSE_CUDA(cudaMemsetAsync(m->vp.ptr, 0, v_bytes, s));
-  m->tiles = DevMem((size_t)m->max_tiles * sizeof(tc::Tile));
-  m->err = DevMem(2 * sizeof(int));
-  BSE_CUDA(cudaMemsetAsync(m->err.ptr, 0, sizeof(int), s));
+  m->vp.reset(new DeviceBuffer(v_bytes, s));
+  BSE_CUDA(cudaMemsetAsync(m->vp->ptr, 0, v_bytes, s));
+  m->err.reset(new DeviceBuffer(2 * sizeof(int), s));
+  BSE_CUDA(cudaMemsetAsync(m->err->ptr, 0, 2 * sizeof(int), s));
   for (int which = 0; which < (B ? 2 : 1); ++which) {
     SplitArgs sa{reinterpret_cast<const double2*>(which ? B : A), SPLIT_DENSE, nullptr, 0, 0, n,
                  m->Kp, n, m->pieces, 1, nullptr,
-                 (which ? m->bp : m->ap).as<__nv_bfloat16>(), n, 0};
+                 (which ? m->bp : m->ap)->as<__nv_bfloat16>(), n, 0};
     sa.src_ld = ld;
     sa.zero_diag = which == 0;
     launch_split(sa, s);
   }
-  m->ma_a = make_plane_map(m->ap.as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
-  if (B) m->ma_b = make_plane_map(m->bp.as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
-  m->mb_v = make_plane_map(m->vp.as<__nv_bfloat16>(), m->Kp, m->kmax_rows,
+  m->ma_a = make_plane_map(m->ap->as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
+  if (B) m->ma_b = make_plane_map(m->bp->as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
+  m->mb_v = make_plane_map(m->vp->as<__nv_bfloat16>(), m->Kp, m->kmax_rows,
                            tc::b_planes(m->pieces), m->nt);
+  matvec_tiles(m.get(), 1, true, s);   // uploaded here: later products may be captured
   return m.release();
 }
+
+namespace {
+// out = (the matrix of map ma) V for the k columns whose planes are in m->vp
+void matvec_block(TcMatvec* m, const CUtensorMap& ma, int k, const double2* diag, const double2* v,
+                  double2* out, cudaStream_t s) {
+  const int ncol = (k + m->nt - 1) / m->nt;
+  if (k <= m->split_cols) {
+    const TcMatvec::TileList& tl = matvec_tiles(m, ncol, true, s);
+    launch_gemm(ma, m->mb_v, tl.dev->as<tc::Tile>(), (int)tl.host.size(), m->sh_seg,
+                MatvecPartEpi{m->part->as<float2>(), m->n, k}, m->err->as<int>(), s, ncol == 1);
+    k_matvec_reduce<<<dim3((m->n + 255) / 256, k), 256, 0, s>>>(
+        m->n, k, m->nseg, m->part->as<float2>(), diag, m->ld, v, out);
+    BSE_CUDA(cudaGetLastError());
+    note_launches(1);
+    return;
+  }
+  const TcMatvec::TileList& tl = matvec_tiles(m, ncol, false, s);
+  launch_gemm(ma, m->mb_v, tl.dev->as<tc::Tile>(), (int)tl.host.size(), m->sh,
+              MatvecEpi{out, m->n, k, diag, m->ld, v}, m->err->as<int>(), s);
+}
+}  // namespace
 
 void tc_matvec_apply(TcMatvec* m, const bse_c128* V, int k, bse_c128* AV, bse_c128* BV,
                      cudaStream_t s) {
   if (k <= 0) return;
   if (k > m->kmax) throw Error(BSE_ERR_UNSUPPORTED, "tensor-core matvec block wider than planned");
   SplitArgs sv{reinterpret_cast<const double2*>(V), SPLIT_DENSE, nullptr, 0, 0, m->n, m->Kp, k,
-               m->pieces, 0, nullptr, m->vp.as<__nv_bfloat16>(), m->kmax_rows, 0};
+               m->pieces, 0, nullptr, m->vp->as<__nv_bfloat16>(), m->kmax_rows, 0};
   sv.bneg = 1;   // the B operand of the matvec GEMMs
   launch_split(sv, s);
-  std::vector<tc::Tile> tl;
-  for (int m0 = 0; m0 < m->n; m0 += tc::BM)
-    for (int n0 = 0; n0 < k; n0 += m->nt)
-      tl.push_back({m0, std::min(tc::BM, m->n - m0), n0, n0, std::min(m->nt, k - n0), m0, 0});
-  BSE_CUDA(cudaMemcpyAsync(m->tiles.ptr, tl.data(), tl.size() * sizeof(tc::Tile),
-                           cudaMemcpyHostToDevice, s));
-  launch_gemm(m->ma_a, m->mb_v, m->tiles.as<tc::Tile>(), (int)tl.size(), m->sh,
-              MatvecEpi{reinterpret_cast<double2*>(AV), m->n, reinterpret_cast<const double2*>(m->A),
-                        m->ld, reinterpret_cast<const double2*>(V)},
-              m->err.as<int>(), s);
+  const double2* v = reinterpret_cast<const double2*>(V);
+  matvec_block(m, m->ma_a, k, reinterpret_cast<const double2*>(m->A), v,
+               reinterpret_cast<double2*>(AV), s);
   if (m->has_b && BV)
-    launch_gemm(m->ma_b, m->mb_v, m->tiles.as<tc::Tile>(), (int)tl.size(), m->sh,
-                MatvecEpi{reinterpret_cast<double2*>(BV), m->n}, m->err.as<int>(), s);
+    matvec_block(m, m->ma_b, k, nullptr, nullptr, reinterpret_cast<double2*>(BV), s);
+}
+
+TcMatvecIo tc_matvec_io(const TcMatvec* m) {
+  return TcMatvecIo{m->vp->ptr, (int64_t)m->kmax_rows * m->Kp, m->pieces, m->nseg,
+                    m->part->as<float2>(), reinterpret_cast<const double2*>(m->A), m->ld};
+}
+
+void tc_matvec_products(TcMatvec* m, cudaStream_t s) {
+  const TcMatvec::TileList& tl = matvec_tiles(m, 1, true, s);
+  launch_gemm(m->ma_a, m->mb_v, tl.dev->as<tc::Tile>(), (int)tl.host.size(), m->sh_seg,
+              MatvecPartEpi{m->part->as<float2>(), m->n, 1}, m->err->as<int>(), s, true);
+}
+
+void tc_matvec_check(TcMatvec* m, cudaStream_t s) {
   int herr = 0;
-  BSE_CUDA(cudaMemcpyAsync(&herr, m->err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
-  BSE_CUDA(cudaStreamSynchronize(s));   // also keeps the host tile list alive until used
+  BSE_CUDA(cudaMemcpyAsync(&herr, m->err->ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
+  BSE_CUDA(cudaStreamSynchronize(s));
   if (herr) throw Error(BSE_ERR_TIMEOUT, "tensor-core matvec: a bounded pipeline wait expired");
 }
 

@@ -427,7 +427,10 @@ struct Solver {
     BSE_CUDA(cudaGetLastError());
     note_launches(1);
     BSE_CUDA(cudaMemcpyAsync(res.data(), nrm.ptr, (size_t)k * 8, cudaMemcpyDeviceToHost, s));
-    BSE_CUDA(cudaStreamSynchronize(s));
+    if (tcm)
+      tc_matvec_check(tcm, s);   // syncs
+    else
+      BSE_CUDA(cudaStreamSynchronize(s));
   }
 };
 

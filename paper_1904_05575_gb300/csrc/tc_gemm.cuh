@@ -211,7 +211,9 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 }
 
 struct GemmShape {    // stages <= 8
-  int nt;          // output columns per tile (multiple of 32, <= 128: 4 accumulators in TMEM)
+  int nt;          // output columns per tile (multiple of 32, <= 128: 4 accumulators in TMEM;
+                   // or 8, whole K only, for products with a single vector: a quarter
+                   // of the column operand's bytes of nt = 32)
   int kchunks;     // padded K / 16
   int pieces;      // BF16 pieces per real number (2 or 3)
   int stages;      // pipeline depth
@@ -584,6 +586,21 @@ gemm_split_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         float re[32], im[32], cr[32], ci[32];
         const uint32_t lane_base =
             tmem_base + (uint32_t)buf * 4u * (uint32_t)sh.nt + ((uint32_t)(quarter * 32) << 16);
+        if (sh.nt == 8) {   // both pairs of accumulators lie in 32 columns
+          if (half == 0) {
+            tmem_ld32(lane_base, cr);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              re[j] = j < 8 ? cr[j % 8] + cr[16 + j % 8] : 0.f;
+              im[j] = j < 8 ? cr[8 + j % 8] + cr[24 + j % 8] : 0.f;
+            }
+            if (row < tl.m_valid) epi(tl, row, 0, re, im);
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&pp.tmem_empty[buf]);
+          continue;
+        }
         for (int c0 = 32 * half; c0 < sh.nt; c0 += 64) {
           tmem_ld32(lane_base + (uint32_t)c0, re);
           tmem_ld32(lane_base + (uint32_t)(sh.nt + c0), im);
