@@ -101,15 +101,28 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& err) 
 namespace bse {
 
 // FP64 (given as its two 32-bit words) -> FP32, round half up, 32-bit
-// integer instructions only.  |x| < 2^-126 becomes a signed zero.
-__device__ __forceinline__ uint32_t f64w_to_f32_bits(uint32_t lo, uint32_t hi) {
-  const uint32_t sign = hi & 0x80000000u;
-  const int e = (int)((hi >> 20) & 0x7FFu);
-  const int be = e - 896;                                     // FP32 biased exponent
-  uint32_t m = ((hi & 0xFFFFFu) << 3) | (lo >> 29);            // top 23 fraction bits
-  uint32_t f = ((uint32_t)be << 23) + m + ((lo >> 28) & 1u);   // rounding carries into the exponent
-  f = be <= 0 ? 0u : (be >= 255 ? 0x7F800000u : f);
-  return sign | f;
+// integer instructions only.  |x| < 2^-126 becomes a signed zero, |x| >= 2^128
+// (and what rounds there) an infinity.  The word shifted left by 3 holds the
+// low 9 exponent bits above the 23 fraction bits, so re-biasing (896 = 384 mod
+// 512) and rounding are one three-operand add.
+__host__ __device__ __forceinline__ uint32_t f64w_to_f32_bits(uint32_t lo, uint32_t hi) {
+  const uint32_t f = ((hi << 3) | (lo >> 29)) - (384u << 23) + ((lo >> 28) & 1u);
+  const uint32_t mag = hi & 0x7FFFFFFFu;
+  const bool in = mag - (897u << 20) < (254u << 20);   // biased FP32 exponent in [1, 254]
+  const uint32_t r = in ? f : mag < (897u << 20) ? 0u : 0x7F800000u;
+  return (hi & 0x80000000u) | r;
+}
+
+// The same where |x| lies in [2^-126, 2^128), without the range check: the
+// caller checks `out` (the largest f64w_range of a group of words) once and
+// converts the group again with the function above if it is not below
+// kF64InRange (zeros and padding).
+constexpr uint32_t kF64InRange = 254u << 20;
+__host__ __device__ __forceinline__ uint32_t f64w_range(uint32_t hi) {
+  return (hi & 0x7FFFFFFFu) - (897u << 20);
+}
+__host__ __device__ __forceinline__ uint32_t f64w_to_f32_in_range(uint32_t lo, uint32_t hi) {
+  return (hi & 0x80000000u) | (((hi << 3) | (lo >> 29)) - (384u << 23) + ((lo >> 28) & 1u));
 }
 
 // FP32 -> BF16 bit pattern, round to nearest even (finite inputs).

@@ -14,7 +14,7 @@
 //                 from A (W^rr) or B (W^ra) in FP64: a tensor-core GEMM per pair
 //                 block where both sides have >= 64 rows, else FP32 on CUDA
 //                 cores reading the complex128 input directly (k_stage2_skinny,
-//                 k_stage2_multi, k_stage2_pipe, k_stage2<TX, TT, RX, RT>)
+//                 k_stage2_multi, k_stage2_pipe, k_stage2<TX, TT, RX, RT>, k_stage2_rows)
 // Where every pair block fits the fused epilogue (rows_t a power of two,
 // rows_x <= min(16, rows_t)), steps 3 and 4 run as one tcgen05 launch whose
 // epilogue performs the contraction on the TMEM tile (tc_direct.cuh).
@@ -291,6 +291,7 @@ struct TOut {
 };
 
 struct TEpiMulti {
+  static constexpr bool kNarrow = false;
   const TOut* outs;
   __device__ __forceinline__ void operator()(const tc::Tile& t, int row, int c0, const float* re,
                                              const float* im) const {
@@ -380,6 +381,7 @@ struct S2TcParams {
 };
 
 struct S2TcEpi {
+  static constexpr bool kNarrow = false;
   const S2TcParams* params;
   __device__ __forceinline__ void operator()(const tc::Tile& t, int row, int c0, const float* re,
                                              const float* im) const {
@@ -709,6 +711,285 @@ __global__ void __launch_bounds__(256) k_stage2_pipe(Stage2Args a) {
   *dst = o;
 }
 
+// One X row per thread against a tile of 2 P rows of T: one or more pair blocks
+// (or an x-row / t-row tile of a large one) per thread block.
+//   - TMA boxes bring the raw complex128 X rows (128-byte swizzle: each thread
+//     reads its own row without bank conflicts) and the FP32 T rows of the next
+//     S2_GC = 8 plane waves into a four-deep ring (zero-filled past NG);
+//   - T is rearranged once per chunk into pairs of neighbouring rows (re0, re1,
+//     im0, im1): one broadcast LDS.128 feeds four packed FMAs;
+//   - a thread converts its X element in registers, where (re, re), (-im, -im)
+//     and (im, im) serve all 2 P outputs;
+//   - the sums of 8 plane waves fold into compensated (hi, lo) pairs (TwoSum).
+// The products, their order and every rounding are those of the one-output
+// kernels below (packed FMAs round each lane like the scalar ones).
+// Bound by latency and issue together (0.4 instructions per clock and
+// scheduler with ten warps per SM at 168 registers; the packed FMA pipe 44 %
+// busy).  4 x 12 bands, NG = 181, 4,096 pairs: W^rr (144 X rows, 16 T rows)
+// 1,453 -> 863 us, W^ra (48 x 48) 1,178 -> 735 us against 32 x 32 tiles with
+// 2 x 2 outputs per thread; 36 x 16 and 25 x 9 blocks (46,656 / 2 pairs, NG =
+// 113) 1,681 -> 1,491 us.  Tried and slower: 4 x 4 packed outputs per thread
+// with X converted through shared memory (861 / 803 us), fewer T rows per
+// thread for more warps (8: 1,159 / 1,043 us), 20 T rows for 40 x 40 blocks.
+constexpr int S2_GC = 8, S2_RING = 4, S2_MAXTH = 160, S2_MAXPB = 8;
+
+struct S2Tile {
+  int npair, pb;             // pair blocks of the launch, per thread block
+  int tx, nxt, tt, ntt;      // x rows per tile and tiles, t rows per tile and tiles
+  int p;                     // T row pairs per thread (the kernel's P, 2 p >= tt)
+  __host__ __device__ int rp() const { return (tx + 7) / 8 * 8; }      // X rows per pair in a slot
+  __host__ __device__ int threads() const { return (pb * tx + 31) / 32 * 32; }
+  // T boxes start at an even row (16-byte aligned), so they hold two rows more
+  __host__ __device__ int tbox() const { return 2 * p + 2; }
+  __host__ __device__ int xslot() const { return pb * rp() * S2_GC * 16; }   // bytes per ring slot
+  __host__ __device__ int tslot() const { return (pb * tbox() * S2_GC * 8 + 127) / 128 * 128; }
+  __host__ __device__ int tpitch() const { return S2_GC * p + 1; }   // float4 per pair: odd, no conflicts
+  __host__ __device__ size_t smem() const {
+    return 1024 + (size_t)S2_RING * (xslot() + tslot()) + 2 * (size_t)pb * tpitch() * 16;
+  }
+};
+
+template <int P>
+__global__ void __launch_bounds__(S2_MAXTH, P <= 4 ? 4 : P <= 6 ? 3 : 2)
+k_stage2_rows(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap tmap,
+              Stage2Args a, S2Tile t, int* err, long long wait) {
+  extern __shared__ uint8_t s2_raw[];
+  __shared__ uint64_t full[S2_RING];
+  __shared__ volatile int abort_flag;
+  __shared__ int xrow[S2_MAXPB], trow[S2_MAXPB];   // first X and T row of each pair
+  __shared__ int64_t ot_s[2 * P];                  // t row part of an output's element of A or B
+  const int xslot = t.xslot(), tslot = t.tslot();
+  constexpr int tbox = 2 * P + 2, tpitch = S2_GC * P + 1;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s2_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint8_t* Xr = smem;                                    // [ring][pair][rp][8] complex128, swizzled
+  uint8_t* Tr = smem + S2_RING * xslot;                  // [ring][pair][8][tbox] float2
+  float4* Tf = reinterpret_cast<float4*>(Tr + S2_RING * tslot);   // [2][pair][8][P] (+1 per pair)
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tiles = t.nxt * t.ntt;
+  const int p0 = blockIdx.x / tiles * t.pb, tile = blockIdx.x % tiles;
+  const int rx0 = tile / t.ntt * t.tx, rt0 = tile % t.ntt * t.tt;
+  const int nrx = min(t.tx, a.rows_x - rx0), nrt = min(t.tt, a.rows_t - rt0);
+  const int npv = min(t.pb, t.npair - p0);   // pairs of this block
+  if (tid < npv) {
+    const int p = s2_pair(a, p0 + tid);
+    const int k = a.k_begin + p / a.nk, kp = p % a.nk;
+    xrow[tid] = (a.x_transpose_pair ? kp * a.nk + k : p) * a.rows_x + rx0;
+    trow[tid] = (int)a.t_row0 + a.slot_of_pair[p] * a.rows_t + rt0;
+  }
+  if (tid == 0) {
+    for (int s = 0; s < S2_RING; ++s) tc::mbar_init(&full[s], 1);
+    abort_flag = 0;
+    tc::fence_barrier_init();
+  }
+  __syncthreads();
+  const int nch = (a.ng + S2_GC - 1) / S2_GC;
+
+  auto fetch = [&](int c) {   // warp 0: the boxes of chunk c into slot c % ring
+    if (c >= nch || tid >= 32) return;
+    const int slot = c % S2_RING;
+    if (tid == 0) tc::mbar_expect_tx(&full[slot], (uint32_t)npv * (t.tx * S2_GC * 16 + tbox * S2_GC * 8));
+    __syncwarp();
+    if (tid < npv) {
+      tc::tma_load_2d(Xr + slot * xslot + tid * t.rp() * S2_GC * 16, &xmap, 2 * S2_GC * c, xrow[tid],
+                      &full[slot]);
+      tc::tma_load_2d(Tr + slot * tslot + tid * tbox * S2_GC * 8, &tmap, 2 * (trow[tid] & ~1),
+                      S2_GC * c, &full[slot]);
+    }
+  };
+  int fetched = min(nch, S2_RING);   // chunks whose copies were issued
+  for (int c = 0; c < S2_RING; ++c) fetch(c);
+
+  // this thread's T row pairs of the rearrangement (at most 4: checked by the host)
+  const float tsign = a.conj_t ? -1.f : 1.f;
+  int toff[4], tdst[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int i = tid + k * nth, q = i / (S2_GC * P), o = i - q * (S2_GC * P), g = o / P, pr = o - g * P;
+    toff[k] = q < npv ? (q * S2_GC + g) * tbox + 2 * pr + (trow[q < npv ? q : 0] & 1) : -1;
+    tdst[k] = q * tpitch + o;
+  }
+  auto convert = [&](int c) {
+    const float2* ts = reinterpret_cast<const float2*>(Tr + c % S2_RING * tslot);
+    float4* td = Tf + (c & 1) * t.pb * tpitch;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (toff[k] >= 0) {
+        const float2 v = ts[toff[k]], w = ts[toff[k] + 1];
+        td[tdst[k]] = make_float4(v.x, w.x, v.y * tsign, w.y * tsign);
+      }
+  };
+  // every thread waits for the chunk's copies; false (in every thread): gave up
+  auto landed = [&](int c) {
+    const bool ok = tc::mbar_wait(&full[c % S2_RING], (c / S2_RING) & 1, &abort_flag, err, wait);
+    return __syncthreads_and(ok) != 0;
+  };
+
+  // this thread's X row, and its and its T rows' parts of the element (al, ap)
+  // of A or B, al + ap ld
+  const int q = tid / t.tx, lx = tid - q * t.tx;
+  const bool active = q < npv && lx < nrx;
+  auto part = [&](bool x, int r) -> int64_t {
+    if (a.mode == S2_RA) {                                // x = (v', c), t = (v, c')
+      const int b = r / a.nc, c = r - b * a.nc;
+      return x ? (int64_t)b * a.nc * a.ld + c : (int64_t)b * a.nc + c * a.ld;
+    }
+    if ((a.mode == S2_RR_CC) == x) {                      // the (v, v') side
+      const int v = r / a.nv, vp = r - v * a.nv;
+      return (int64_t)v * a.nc + (int64_t)vp * a.nc * a.ld;
+    }
+    const int c = r / a.nc, cp = r - c * a.nc;            // the (c, c') side
+    return c + cp * a.ld;
+  };
+  const int64_t o0 = part(true, rx0 + lx);
+  for (int i = tid; i < nrt; i += nth) ot_s[i] = part(false, rt0 + i);
+  const uint32_t xoff = active ? (q * t.rp() + lx) * (S2_GC * 16) + (lx & 7) * 16 : 0;
+  const int tq = active ? q * tpitch : 0;
+  const uint32_t xflip = a.conj_x ? 0x80000000u : 0u;
+  uint64_t HX[P], HY[P], LX[P], LY[P];
+#pragma unroll
+  for (int j = 0; j < P; ++j) HX[j] = HY[j] = LX[j] = LY[j] = 0ull;
+
+  bool ok_all = landed(0);
+  if (ok_all) convert(0);
+  for (int c = 0; c < nch; ++c) {
+    // T of chunk c rearranged and chunk c - 1 consumed by every thread: its
+    // ring slot takes chunk c + 2
+    if (c + 1 < nch) {
+      ok_all = ok_all && landed(c + 1);
+      if (!ok_all) break;
+      if (c > 0) {
+        fetch(c - 1 + S2_RING);
+        fetched = min(nch, c + S2_RING);
+      }
+      convert(c + 1);
+    } else {
+      __syncthreads();
+    }
+    const uint8_t* xs = Xr + c % S2_RING * xslot;
+    const float4* tf = Tf + (c & 1) * t.pb * tpitch + tq;
+    uint64_t ax[P], ay[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j) ax[j] = ay[j] = 0ull;
+    // the chunk's X elements, with one range check for all eight (a branch per
+    // element kept the conversions from overlapping the FMAs)
+    uint32_t xre[S2_GC], xim[S2_GC], range = 0u;
+#pragma unroll
+    for (int g = 0; g < S2_GC; ++g) {
+      const uint4 d = *reinterpret_cast<const uint4*>(xs + (xoff ^ (g * 16)));
+      range = max(range, max(f64w_range(d.y), f64w_range(d.w)));
+      xre[g] = f64w_to_f32_in_range(d.x, d.y);
+      xim[g] = f64w_to_f32_in_range(d.z, d.w) ^ xflip;
+    }
+    if (range >= kF64InRange) {
+#pragma unroll 1
+      for (int g = 0; g < S2_GC; ++g) {
+        const uint4 d = *reinterpret_cast<const uint4*>(xs + (xoff ^ (g * 16)));
+        const uint32_t re = f64w_to_f32_bits(d.x, d.y), im = f64w_to_f32_bits(d.z, d.w) ^ xflip;
+#pragma unroll
+        for (int u = 0; u < S2_GC; ++u)
+          if (u == g) {
+            xre[u] = re;
+            xim[u] = im;
+          }
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < S2_GC; ++g) {
+      const uint32_t re = xre[g], im = xim[g];
+      const uint64_t xr = ((uint64_t)re << 32) | re, xi = ((uint64_t)im << 32) | im;
+      const uint64_t xn = xi ^ 0x8000000080000000ull;
+      // (groups of 4 pairs, each step over the whole group: the second FMA of
+      // a sum is eight instructions behind the first)
+#pragma unroll
+      for (int j0 = 0; j0 < P; j0 += 4) {
+        ulonglong2 tv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j0 + j < P) tv[j] = *reinterpret_cast<const ulonglong2*>(tf + g * P + j0 + j);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j0 + j < P) ax[j0 + j] = tc::ffma2(xr, tv[j].x, ax[j0 + j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j0 + j < P) ay[j0 + j] = tc::ffma2(xr, tv[j].y, ay[j0 + j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j0 + j < P) ax[j0 + j] = tc::ffma2(xn, tv[j].y, ax[j0 + j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j0 + j < P) ay[j0 + j] = tc::ffma2(xi, tv[j].x, ay[j0 + j]);
+      }
+    }
+    tc::two_sum2_all<P>(HX, LX, ax);
+    tc::two_sum2_all<P>(HY, LY, ay);
+  }
+  if (!ok_all) {   // let the copies issued land before shared memory goes away
+    if (tid == 0) {
+      const long long t0 = clock64();
+      for (int c = max(0, fetched - S2_RING); c < fetched; ++c)
+        while (!tc::mbar_try_wait(&full[c % S2_RING], (c / S2_RING) & 1) &&
+               clock64() - t0 < tc::WAIT_CYCLES) {
+        }
+    }
+    return;
+  }
+  if (!active) return;
+  const int p = s2_pair(a, p0 + q);
+  const int k = a.k_begin + p / a.nk, kp = p % a.nk;
+  double2* out = a.out + ((int64_t)k + (int64_t)kp * a.ld) * a.nv * a.nc + o0;
+  const float sc = (float)a.scale;
+#pragma unroll
+  for (int j0 = 0; j0 < P; j0 += 2) {   // four outputs at a time: the loads, then the stores
+    double2 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (2 * j0 + u < nrt && j0 + u / 2 < P) v[u] = out[ot_s[2 * j0 + u]];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + u / 2 < P && 2 * j0 + u < nrt) {
+        const int j = j0 + u / 2 < P ? j0 + u / 2 : 0;
+        const uint64_t hx = HX[j], lx2 = LX[j], hy = HY[j], ly = LY[j];
+        // contribution formed in FP32 (hi + lo carries the compensated sum), widened exactly
+        double2 w = v[u];
+        w.x -= f32_to_f64_bits(u & 1 ? scale_hi_lo(sc, tc::hi_of(hx), tc::hi_of(lx2))
+                                     : scale_hi_lo(sc, tc::lo_of(hx), tc::lo_of(lx2)));
+        w.y -= f32_to_f64_bits(u & 1 ? scale_hi_lo(sc, tc::hi_of(hy), tc::hi_of(ly))
+                                     : scale_hi_lo(sc, tc::lo_of(hy), tc::lo_of(ly)));
+        out[ot_s[2 * j0 + u]] = w;
+      }
+  }
+}
+
+// Tile of k_stage2_rows for a pair block: t rows in equal tiles of at most 16
+// (P = 8: 96 registers of accumulators), x rows in equal tiles of at most
+// S2_MAXTH, and as many pairs per block as fill its warps best.
+S2Tile stage2_tile(const Stage2Args& a, int npair) {
+  auto up = [](int x, int m) { return (x + m - 1) / m; };
+  S2Tile t{};
+  t.npair = npair;
+  t.ntt = up(a.rows_t, 16);
+  t.tt = up(a.rows_t, t.ntt);
+  for (int p : {4, 6, 8})
+    if (!t.p && 2 * p >= t.tt) t.p = p;
+  t.nxt = up(a.rows_x, S2_MAXTH);
+  t.tx = up(a.rows_x, t.nxt);
+  t.pb = 1;
+  if (t.nxt == 1) {
+    double best = 0.0;
+    for (int pb = 1; pb <= S2_MAXPB && pb * t.tx <= S2_MAXTH; ++pb) {
+      const int th = up(pb * t.tx, 32) * 32;
+      if (pb * S2_GC * t.p > 4 * th) break;       // T pairs per thread of the rearrangement
+      const double fill = (double)(pb * t.tx) / th;
+      if (fill > best + 0.02 || (th <= 96 && fill > best - 0.05)) {   // (blocks of 3 warps or more)
+        best = std::max(best, fill);
+        t.pb = pb;
+      }
+    }
+  }
+  return t;
+}
+
 // Stage 2 for skinny pair blocks: at most RT rows of T against X rows of 16
 // or more (W^rr with 2 core levels: 4 (v, v') rows of T, 400 (c, c') rows of
 // X; or 2 conduction bands against 4 to 6 valence bands).  One
@@ -996,29 +1277,65 @@ __global__ void __launch_bounds__(256) k_stage2_multi(Stage2Args a, int npair, i
   *dst = o2;
 }
 
-// The kernel whose tile fits the pair block best (every variant adds in the
-// same order: the results do not depend on the choice).
-void launch_stage2(const Stage2Args& a, int npair, cudaStream_t s) {
-  if (stage2_skinny(a)) {
-    const int64_t total = (int64_t)npair * a.rows_x;
-    const int64_t blocks = (total + SK_ROWS - 1) / SK_ROWS;
-    k_stage2_skinny<4><<<(unsigned)blocks, SK_ROWS, 0, s>>>(a, total);
-  } else if (a.rows_x <= 16 && a.rows_t <= 16) {
-    const int pb = stage2_multi_pairs(a);
-    if (pb >= 2)
+struct S2Maps {   // k_stage2_rows: the tile and the tensor maps of its boxes
+  S2Tile tile;
+  CUtensorMap x, t;
+};
+
+// The kernel for the pair block (every variant adds in the same order: the
+// results do not depend on the choice).
+enum Stage2Form { S2F_SKINNY, S2F_MULTI, S2F_PIPE, S2F_24, S2F_40, S2F_ROWS };
+Stage2Form stage2_form(const Stage2Args& a) {
+  // one X row per thread where T has at most 4 rows (bound by reading X once)
+  if (stage2_skinny(a)) return S2F_SKINNY;
+  // one output per thread where two whole blocks fit 256 threads that way, or one to 16 x 16
+  if (stage2_multi_pairs(a) >= 2) return S2F_MULTI;
+  if (a.rows_x <= 16 && a.rows_t <= 16) return S2F_PIPE;
+  // nearly square blocks that one tile of 2 x 3 or 2 x 5 outputs per thread
+  // covers: 24 x 24 (with 15 x 15 and 4 x 4: 1,231 us against 1,465 us for
+  // k_stage2_rows), 40 x 40 (755 against 974 us); with T rows for at most one
+  // k_stage2_rows tile that form is the faster one (36 x 16, 25 x 9)
+  if (a.rows_t > 16 && a.rows_x <= 24 && a.rows_t <= 24) return S2F_24;
+  if (a.rows_t > 24 && a.rows_x <= 40 && a.rows_t <= 40) return S2F_40;
+  return S2F_ROWS;
+}
+
+void launch_stage2(const Stage2Args& a, int npair, const S2Maps& m, int* err, long long wait,
+                   cudaStream_t s) {
+  switch (stage2_form(a)) {
+    case S2F_SKINNY: {
+      const int64_t total = (int64_t)npair * a.rows_x;
+      const int64_t blocks = (total + SK_ROWS - 1) / SK_ROWS;
+      k_stage2_skinny<4><<<(unsigned)blocks, SK_ROWS, 0, s>>>(a, total);
+      break;
+    }
+    case S2F_MULTI: {
+      const int pb = stage2_multi_pairs(a);
       k_stage2_multi<<<(npair + pb - 1) / pb, 256, 0, s>>>(a, npair, pb);
-    else
-      k_stage2_pipe<<<npair, 256, 0, s>>>(a);
-  } else if (a.rows_x <= 24 && a.rows_t <= 24) {           // e.g. W^ra, 4 x 6 bands
-    launch_stage2_tiles<24, 24, 2, 3>(a, npair, s);
-  } else if (a.rows_x <= 32 && a.rows_t <= 16) {           // e.g. W^rr, 3 x 5 bands (25 x 9)
-    launch_stage2_tiles<32, 16, 2, 2>(a, npair, s);
-  } else if (a.rows_x <= 40 && a.rows_t <= 16) {           // e.g. W^rr, 4 x 6 bands (36 x 16)
-    launch_stage2_tiles<40, 16, 2, 2>(a, npair, s);
-  } else if (a.rows_x <= 40 && a.rows_t <= 40) {           // e.g. W^ra, 2 x 20 bands (40 x 40)
-    launch_stage2_tiles<40, 40, 2, 5>(a, npair, s);
-  } else {
-    launch_stage2_tiles<32, 32, 2, 2>(a, npair, s);
+      break;
+    }
+    case S2F_PIPE: k_stage2_pipe<<<npair, 256, 0, s>>>(a); break;
+    case S2F_24: launch_stage2_tiles<24, 24, 2, 3>(a, npair, s); break;
+    case S2F_40: launch_stage2_tiles<40, 40, 2, 5>(a, npair, s); break;
+    case S2F_ROWS: {
+      const S2Tile& t = m.tile;
+      const int64_t blocks = (int64_t)((npair + t.pb - 1) / t.pb) * t.nxt * t.ntt;
+      auto launch = [&](auto kern) {
+        kern<<<(unsigned)blocks, t.threads(), t.smem(), s>>>(m.x, m.t, a, t, err, wait);
+      };
+      // the shared-memory opt-in, once (launches may be captured)
+      static std::once_flag once;
+      std::call_once(once, [] {
+        for (auto kern : {k_stage2_rows<4>, k_stage2_rows<6>, k_stage2_rows<8>})
+          BSE_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+      });
+      switch (t.p) {
+        case 4: launch(k_stage2_rows<4>); break;
+        case 6: launch(k_stage2_rows<6>); break;
+        default: launch(k_stage2_rows<8>); break;
+      }
+      break;
+    }
   }
   BSE_CUDA(cudaGetLastError());
   note_launches(1);
@@ -1054,6 +1371,23 @@ CUtensorMap make_plane_map(const __nv_bfloat16* base, int Kp, int rows, int plan
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS)
     throw Error(BSE_ERR_CUDA, "cuTensorMapEncodeTiled failed with " + std::to_string((int)r));
+  return m;
+}
+
+// 2-D map over rows of `cols` numbers of `bytes` bytes, `ld_bytes` apart, box {box_cols, box_rows}
+CUtensorMap make_2d_map(const void* base, CUtensorMapDataType type, int64_t cols, int64_t rows,
+                        int64_t ld_bytes, int box_cols, int box_rows,
+                        CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE) {
+  CUtensorMap m;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)ld_bytes};
+  cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = encode_fn()(&m, type, 2, (void*)base, dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    throw Error(BSE_ERR_CUDA, "cuTensorMapEncodeTiled (2-D) failed with " + std::to_string((int)r));
   return m;
 }
 
@@ -1271,6 +1605,7 @@ struct ExParams {
 };
 
 struct ExchangeBatchEpi {   // ExchangeEpi with per-problem outputs
+  static constexpr bool kNarrow = false;
   const ExParams* params;
   __device__ __forceinline__ void operator()(const tc::Tile& t, int row, int c0, const float* re,
                                              const float* im) const {
@@ -1316,6 +1651,7 @@ struct BatchPlan {
     bool w_conj_transpose = false;
     DevMem perm, slot;
     Stage2Args s2{};
+    S2Maps s2maps{};         // its CUDA-core form's tile and tensor maps
     std::vector<int32_t> qh;   // q index of each pair built, in pair-list order
     std::vector<int> act_h;    // the pairs built: every pair of the slab, or k <= k'
     std::vector<int> slot_h;   // pair -> stage-1 slot (-1: not built)
@@ -1466,7 +1802,7 @@ void plan_execute_mixed(BatchPlan& pl, cudaStream_t s) {
         for (BatchPlan::Term& t : pl.terms) {
           if (t.tc2) continue;
           Phase pt(t.s2.mode == S2_RA ? "mixed_stage2_wra" : "mixed_stage2_wrr", s);
-          launch_stage2(t.s2, t.nact, s);
+          launch_stage2(t.s2, t.nact, t.s2maps, pl.err.as<int>(), pl.wait, s);
         }
       }
       if (pl.n_s2tiles || pl.n_s2tiles_t) {
@@ -1880,17 +2216,8 @@ BatchPlan* plan_create(std::vector<Problem> probs, int precision, int flags, cud
         const Stage2Args& a = t.s2;
         const Problem& pr = pl->probs[t.prob];
         const int64_t x_pairs = a.x_transpose_pair ? (int64_t)pr.p.nk * pr.p.nk : pr.slab_pairs();
-        CUtensorMap m;
-        cuuint64_t dims[2] = {(cuuint64_t)2 * a.ng, (cuuint64_t)(x_pairs * a.rows_x)};
-        cuuint64_t strides[1] = {(cuuint64_t)a.ng * 16};
-        cuuint32_t box[2] = {(cuuint32_t)(2 * tc::S2_GB), (cuuint32_t)a.rows_x};
-        cuuint32_t estr[2] = {1, 1};
-        CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, (void*)a.x, dims, strides,
-                                 box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS)
-          throw Error(BSE_ERR_CUDA, "cuTensorMapEncodeTiled (pair side) failed with " + std::to_string((int)r));
-        maps.push_back(m);
+        maps.push_back(make_2d_map(a.x, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2 * a.ng,
+                                   x_pairs * a.rows_x, (int64_t)a.ng * 16, 2 * tc::S2_GB, a.rows_x));
       }
       pl->xmaps = upload_mem(maps);
       for (size_t ti = 0; ti < pl->terms.size(); ++ti) {
@@ -1930,12 +2257,25 @@ BatchPlan* plan_create(std::vector<Problem> probs, int precision, int flags, cud
         any_tc2 = any_tc2 || t.tc2;
         any_fp32 = any_fp32 || !t.tc2;
       }
-      if (any_fp32) pl->tbuf = DevMem((size_t)pl->ng_pad * pl->a_rows * sizeof(float2));
+      const int64_t t_ld = (pl->a_rows + 1) / 2 * 2;   // T rows of 16-byte multiples (tensor map)
+      if (any_fp32) pl->tbuf = DevMem((size_t)pl->ng_pad * t_ld * sizeof(float2));
       std::vector<TOut> outs;
       for (BatchPlan::Term& t : pl->terms) {
         t.s2.T = pl->tbuf.as<float2>();
-        t.s2.t_ld = pl->a_rows;
-        outs.push_back(TOut{t.tc2 ? nullptr : pl->tbuf.as<float2>(), pl->a_rows, nullptr,
+        t.s2.t_ld = t_ld;
+        if (!t.tc2 && stage2_form(t.s2) == S2F_ROWS) {
+          const Stage2Args& a = t.s2;
+          const Problem& pr = pl->probs[t.prob];
+          const int64_t x_pairs = a.x_transpose_pair ? (int64_t)pr.p.nk * pr.p.nk : pr.slab_pairs();
+          S2Maps& m = t.s2maps;
+          m.tile = stage2_tile(a, t.nact);
+          m.x = make_2d_map(a.x, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2 * (int64_t)a.ng,
+                            x_pairs * a.rows_x, (int64_t)a.ng * 16, 2 * S2_GC, m.tile.tx,
+                            CU_TENSOR_MAP_SWIZZLE_128B);
+          m.t = make_2d_map(a.T, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2 * t_ld, a.ng, t_ld * 8,
+                            2 * m.tile.tbox(), S2_GC);
+        }
+        outs.push_back(TOut{t.tc2 ? nullptr : pl->tbuf.as<float2>(), t_ld, nullptr,
                             pl->a_rows, pl->Kp, pl->pieces, t.s2.conj_t});
       }
       if (any_tc2) {
@@ -2178,6 +2518,7 @@ void build_mixed_batch(const std::vector<Problem>& probs, int precision, cudaStr
 // ---------------------------------------------------------------------------
 namespace {
 struct MatvecEpi {
+  static constexpr bool kNarrow = false;
   double2* out;
   int64_t ld;
   int ncols;                       // columns of the block
@@ -2206,6 +2547,7 @@ struct MatvecEpi {
 
 // One K segment's sums of a tile (Tile::prob = segment), [segment][column][row].
 struct MatvecPartEpi {
+  static constexpr bool kNarrow = true;   // tiles of 8 columns too (a single vector)
   float2* part;
   int64_t n;
   int ncols;
@@ -2409,6 +2751,7 @@ namespace {
 constexpr int RPA_KSTEPS = 32;   // K steps per tile (512 transitions)
 
 struct RpaPartialEpi {
+  static constexpr bool kNarrow = false;
   float2* part;   // [splits][ng][ng] row-major partial sums
   int ng;
   __device__ __forceinline__ void operator()(const tc::Tile& t, int row, int c0, const float* re,

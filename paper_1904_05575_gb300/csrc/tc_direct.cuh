@@ -122,6 +122,45 @@ __device__ __forceinline__ void two_sum2(uint64_t& h, uint64_t& l, uint64_t a) {
   l = fadd2(l, e);
 }
 
+// a - b as one FMA with -1 (the same rounding): the packed subtraction takes
+// two sign flips on the integer pipe besides its add
+__device__ __forceinline__ uint64_t fsub2_fma(uint64_t a, uint64_t b) {
+  return ffma2(b, 0xBF800000BF800000ull, a);
+}
+// the same for N sums, four at a time step by step (each step's operands are
+// four instructions old)
+template <int N>
+__device__ __forceinline__ void two_sum2_all(uint64_t (&h)[N], uint64_t (&l)[N], const uint64_t (&a)[N]) {
+#pragma unroll
+  for (int i0 = 0; i0 < N; i0 += 4) {
+    uint64_t sm[4], bp[4], e[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i0 + i < N) sm[i] = fadd2(h[i0 + i], a[i0 + i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i0 + i < N) bp[i] = fsub2_fma(sm[i], h[i0 + i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i0 + i < N) e[i] = fsub2_fma(sm[i], bp[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i0 + i < N) e[i] = fsub2_fma(h[i0 + i], e[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i0 + i < N) bp[i] = fsub2_fma(a[i0 + i], bp[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i0 + i < N) e[i] = fadd2(e[i], bp[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i0 + i < N) {
+        h[i0 + i] = sm[i];
+        l[i0 + i] = fadd2(l[i0 + i], e[i]);
+      }
+  }
+}
+
 // 8 columns of T for this thread's lane: main + correction, real and imaginary
 // (four loads and their wait in one statement, so no use can precede the wait).
 __device__ __forceinline__ void tmem_ld_t8(uint32_t taddr, uint32_t nt, float* tr, float* ti) {

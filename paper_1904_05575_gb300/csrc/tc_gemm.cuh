@@ -445,7 +445,8 @@ __device__ __forceinline__ void mma_role(const Pipe& pp, uint32_t tmem_base, int
 
 // ---------------------------------------------------------------------------
 // The kernel.  Epi provides: __device__ void operator()(const Tile&, int row,
-// int col0, const float* re, const float* im) const  for 32 columns at col0.
+// int col0, const float* re, const float* im) const  for 32 columns at col0,
+// and kNarrow: tiles may have nt = 8 (8 valid columns then).
 // SEG: tiles accumulate K in sh.ksegs segments (compiled only where used, so
 // the register arrays of the segment sums cost nothing elsewhere).
 // units_taken: a device counter zeroed before the launch (dynamic hand-out of
@@ -586,20 +587,22 @@ gemm_split_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         float re[32], im[32], cr[32], ci[32];
         const uint32_t lane_base =
             tmem_base + (uint32_t)buf * 4u * (uint32_t)sh.nt + ((uint32_t)(quarter * 32) << 16);
-        if (sh.nt == 8) {   // both pairs of accumulators lie in 32 columns
-          if (half == 0) {
-            tmem_ld32(lane_base, cr);
+        if constexpr (Epi::kNarrow) {
+          if (sh.nt == 8) {   // both pairs of accumulators lie in 32 columns
+            if (half == 0) {
+              tmem_ld32(lane_base, cr);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              re[j] = j < 8 ? cr[j % 8] + cr[16 + j % 8] : 0.f;
-              im[j] = j < 8 ? cr[8 + j % 8] + cr[24 + j % 8] : 0.f;
+              for (int j = 0; j < 32; ++j) {
+                re[j] = j < 8 ? cr[j % 8] + cr[16 + j % 8] : 0.f;
+                im[j] = j < 8 ? cr[8 + j % 8] + cr[24 + j % 8] : 0.f;
+              }
+              if (row < tl.m_valid) epi(tl, row, 0, re, im);
             }
-            if (row < tl.m_valid) epi(tl, row, 0, re, im);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&pp.tmem_empty[buf]);
+            continue;
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&pp.tmem_empty[buf]);
-          continue;
         }
         for (int c0 = 32 * half; c0 < sh.nt; c0 += 64) {
           tmem_ld32(lane_base + (uint32_t)c0, re);
