@@ -48,7 +48,7 @@ namespace {
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // ---------------------------------------------------------------------------
-// split: one thread per (output row, k); P pieces per real number
+// split: complex rows -> BF16 planes, P pieces per real number
 // ---------------------------------------------------------------------------
 enum SplitMode { SPLIT_DENSE = 0, SPLIT_PAIRS = 1, SPLIT_W = 2 };
 
@@ -76,67 +76,94 @@ struct SplitArgs {
   int64_t src_ld = 0;       // SPLIT_DENSE: source row stride (0: K)
   int zero_diag = 0;        // SPLIT_DENSE: element k == row stored as zero
   int bneg = 0;             // B-operand layout: 3P planes (-Im, Re, Im) per piece
-  int tdense = 0;           // SPLIT_DENSE read transposed: row r, element k at src[k * src_ld + r]
   int c64 = 0;              // src holds complex64 (float re, im) instead of complex128
 };
 
-// One thread per (output row, 8 consecutive k): every element is read as two
+// Every job of a launch in one grid (a plan has up to three per direct term and
+// two per exchange, several of them a few microseconds long: five launches for
+// one small problem took 25 us).
+constexpr int kSplitJobs = 24;
+struct SplitJobs {
+  int njobs = 0;
+  int64_t first[kSplitJobs + 1];   // first block of each job, then the grid
+  uint32_t magic[kSplitJobs];      // ceil(2^32 / (Kp / 4))
+  SplitArgs job[kSplitJobs];
+};
+constexpr int kSplitUnits = 4;     // units of 4 elements per thread
+
+// One thread per unit of 4 consecutive k of a row: every element is read as two
 // 32-bit words, rounded to FP32 with integer instructions and split in FP32
-// into P BF16 pieces; each plane gets one 16-byte store of 8 pieces.
+// into P BF16 pieces; each plane gets one 8-byte store.  Bound by HBM: a warp
+// reads 2 KB and writes 256 bytes per plane, contiguous (units of 8 elements
+// and 16-byte stores touched a 128-byte line per lane and load: c3-like
+// windows 1,295 us, here 930).
 template <int P>
-__global__ void __launch_bounds__(256) k_split(SplitArgs a) {
-  const int kg = a.Kp / 8;
-  const int64_t total = (int64_t)a.rows * kg;
+__global__ void __launch_bounds__(256) k_split(const __grid_constant__ SplitJobs jobs) {
+  int ji = 0;
+  while (ji + 1 < jobs.njobs && (int64_t)blockIdx.x >= jobs.first[ji + 1]) ++ji;
+  const SplitArgs& a = jobs.job[ji];
+  const int kg = a.Kp / 4;
   const int64_t plane = (a.plane_rows ? a.plane_rows : (int64_t)a.rows) * a.Kp;
   const uint4* src = reinterpret_cast<const uint4*>(a.src);   // one complex128 per uint4
   const uint2* src64 = reinterpret_cast<const uint2*>(a.src);  // or one complex64 per uint2
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int row = (int)(i / kg), k0 = (int)(i % kg) * 8;
+  const int64_t u0 = ((int64_t)blockIdx.x - jobs.first[ji]) * (256 * kSplitUnits);
+  const int64_t rbase = u0 / kg;
+  const uint32_t rem = (uint32_t)(u0 - rbase * kg);
+#pragma unroll 2
+  for (int it = 0; it < kSplitUnits; ++it) {
+    const uint32_t v = rem + threadIdx.x + 256 * it;   // < kg + 1,024
+    // v / kg by the reciprocal (exact: v kg < 2^32; 0 where it would not be)
+    const uint32_t dr = jobs.magic[ji] ? __umulhi(v, jobs.magic[ji]) : v / kg;
+    const int64_t row64 = rbase + dr;
+    if (row64 >= a.rows) break;
+    const int row = (int)row64, k0 = (int)(v - dr * kg) * 4;
     int64_t off = (int64_t)row * (a.src_ld ? a.src_ld : a.K), kstride = 1;
-    if (a.tdense) {   // consecutive threads on consecutive rows: coalesced reads
-      row = (int)(i % a.rows);
-      k0 = (int)(i / a.rows) * 8;
-      off = row;
-      kstride = a.src_ld;
-    }
     if (a.mode == SPLIT_PAIRS) {
       const int slot = row / a.rows_per;
-      int j = row % a.rows_per;
+      int j = row - slot * a.rows_per;
       if (a.pair_nb) j = (j % a.pair_nb) * a.pair_nb + j / a.pair_nb;
       off = ((int64_t)a.perm[slot] * a.rows_per + j) * a.K;
     } else if (a.mode == SPLIT_W) {
-      const int q = row / a.rows_per, g = row % a.rows_per;
+      const int q = row / a.rows_per, g = row - q * a.rows_per;
       off = g >= a.K ? -1 : (int64_t)q * a.K * a.K + (a.transpose ? g : (int64_t)g * a.K);
       kstride = a.transpose ? a.K : 1;
     }
-    uint32_t hr[P][8], hi[P][8];
+    uint32_t hr[P][4], hi[P][4];
+    uint32_t fr[4], fi[4];
+    if (a.c64) {   // already FP32
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int k = k0 + e;
-      const bool take = k < a.K && off >= 0 && !(a.zero_diag && k == row);
-      uint32_t fr = 0u, fi = 0u;
-      if (a.c64) {   // already FP32
-        if (take) {
-          const uint2 x = __ldg(src64 + off + (int64_t)k * kstride);
-          fr = x.x;
-          fi = x.y;
-        }
-      } else {
-        uint4 x = make_uint4(0u, 0u, 0u, 0u);
-        if (take) x = __ldg(src + off + (int64_t)k * kstride);
-        fr = f64w_to_f32_bits(x.x, x.y);
-        fi = f64w_to_f32_bits(x.z, x.w);
+      for (int e = 0; e < 4; ++e) {
+        const int k = k0 + e;
+        uint2 x = make_uint2(0u, 0u);
+        if (k < a.K && off >= 0 && !(a.zero_diag && k == row)) x = __ldg(src64 + off + (int64_t)k * kstride);
+        fr[e] = x.x;
+        fi[e] = x.y;
       }
-      if (a.kscale && k < a.K) {   // exchange operand only: scale in FP32
-        const float sc = (float)a.kscale[k];
-        fr = __float_as_uint(__uint_as_float(fr) * sc);
-        fi = __float_as_uint(__uint_as_float(fi) * sc);
+    } else {
+      uint4 x[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int k = k0 + e;
+        x[e] = make_uint4(0u, 0u, 0u, 0u);
+        if (k < a.K && off >= 0 && !(a.zero_diag && k == row)) x[e] = __ldg(src + off + (int64_t)k * kstride);
       }
-      if (a.conj) fi ^= 0x80000000u;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        fr[e] = f64w_to_f32_bits(x[e].x, x[e].y);
+        fi[e] = f64w_to_f32_bits(x[e].z, x[e].w);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (a.kscale && k0 + e < a.K) {   // exchange operand only: scale in FP32
+        const float sc = (float)a.kscale[k0 + e];
+        fr[e] = __float_as_uint(__uint_as_float(fr[e]) * sc);
+        fi[e] = __float_as_uint(__uint_as_float(fi[e]) * sc);
+      }
+      if (a.conj) fi[e] ^= 0x80000000u;
       uint32_t tr[P], ti[P];
-      split_f32_bf16<P>(fr, tr);
-      split_f32_bf16<P>(fi, ti);
+      split_f32_bf16<P>(fr[e], tr);
+      split_f32_bf16<P>(fi[e], ti);
 #pragma unroll
       for (int p = 0; p < P; ++p) {
         hr[p][e] = tr[p];
@@ -146,36 +173,47 @@ __global__ void __launch_bounds__(256) k_split(SplitArgs a) {
     const int64_t o = (a.row0 + row) * a.Kp + k0;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-      uint4 vr, vi;
-      vr.x = hr[p][0] | (hr[p][1] << 16); vr.y = hr[p][2] | (hr[p][3] << 16);
-      vr.z = hr[p][4] | (hr[p][5] << 16); vr.w = hr[p][6] | (hr[p][7] << 16);
-      vi.x = hi[p][0] | (hi[p][1] << 16); vi.y = hi[p][2] | (hi[p][3] << 16);
-      vi.z = hi[p][4] | (hi[p][5] << 16); vi.w = hi[p][6] | (hi[p][7] << 16);
+      const uint2 vr = make_uint2(hr[p][0] | (hr[p][1] << 16), hr[p][2] | (hr[p][3] << 16));
+      const uint2 vi = make_uint2(hi[p][0] | (hi[p][1] << 16), hi[p][2] | (hi[p][3] << 16));
       if (a.bneg) {   // planes 3p: -Im (both BF16 signs flipped), 3p + 1: Re, 3p + 2: Im
-        const uint4 vn = make_uint4(vi.x ^ 0x80008000u, vi.y ^ 0x80008000u, vi.z ^ 0x80008000u,
-                                    vi.w ^ 0x80008000u);
-        *reinterpret_cast<uint4*>(a.out + (int64_t)(3 * p) * plane + o) = vn;
-        *reinterpret_cast<uint4*>(a.out + (int64_t)(3 * p + 1) * plane + o) = vr;
-        *reinterpret_cast<uint4*>(a.out + (int64_t)(3 * p + 2) * plane + o) = vi;
+        const uint2 vn = make_uint2(vi.x ^ 0x80008000u, vi.y ^ 0x80008000u);
+        *reinterpret_cast<uint2*>(a.out + (int64_t)(3 * p) * plane + o) = vn;
+        *reinterpret_cast<uint2*>(a.out + (int64_t)(3 * p + 1) * plane + o) = vr;
+        *reinterpret_cast<uint2*>(a.out + (int64_t)(3 * p + 2) * plane + o) = vi;
       } else {
-        *reinterpret_cast<uint4*>(a.out + (int64_t)p * plane + o) = vr;
-        *reinterpret_cast<uint4*>(a.out + (int64_t)(P + p) * plane + o) = vi;
+        *reinterpret_cast<uint2*>(a.out + (int64_t)p * plane + o) = vr;
+        *reinterpret_cast<uint2*>(a.out + (int64_t)(P + p) * plane + o) = vi;
       }
     }
   }
 }
 
-void launch_split(const SplitArgs& a, cudaStream_t s) {
-  const int64_t total = (int64_t)a.rows * (a.Kp / 8);
-  int64_t blocks = (total + 255) / 256;
-  if (blocks > 152 * 32) blocks = 152 * 32;
-  if (a.pieces == 3)
-    k_split<3><<<(int)std::max<int64_t>(blocks, 1), 256, 0, s>>>(a);
-  else
-    k_split<2><<<(int)std::max<int64_t>(blocks, 1), 256, 0, s>>>(a);
-  BSE_CUDA(cudaGetLastError());
-  note_launches(1);
+void launch_splits(const std::vector<SplitArgs>& all, cudaStream_t s) {
+  for (size_t j0 = 0; j0 < all.size(); j0 += kSplitJobs) {
+    SplitJobs jobs;
+    int64_t blocks = 0;
+    for (size_t j = j0; j < std::min(all.size(), j0 + kSplitJobs); ++j) {
+      const SplitArgs& a = all[j];
+      const int64_t units = (int64_t)a.rows * (a.Kp / 4), per = 256 * kSplitUnits;
+      if (blocks + units / per >= INT32_MAX) throw Error(BSE_ERR_UNSUPPORTED, "split: too many rows");
+      jobs.first[jobs.njobs] = blocks;
+      jobs.magic[jobs.njobs] =
+          a.Kp / 4 < 1 << 15 ? (uint32_t)(((1ull << 32) + a.Kp / 4 - 1) / (a.Kp / 4)) : 0u;
+      jobs.job[jobs.njobs++] = a;
+      blocks += (units + per - 1) / per;
+    }
+    jobs.first[jobs.njobs] = blocks;
+    if (blocks == 0) continue;
+    if (jobs.job[0].pieces == 3)
+      k_split<3><<<(unsigned)blocks, 256, 0, s>>>(jobs);
+    else
+      k_split<2><<<(unsigned)blocks, 256, 0, s>>>(jobs);
+    BSE_CUDA(cudaGetLastError());
+    note_launches(1);
+  }
 }
+
+void launch_split(const SplitArgs& a, cudaStream_t s) { launch_splits({a}, s); }
 
 // ---------------------------------------------------------------------------
 // epilogues of the tensor-core GEMM
@@ -1710,6 +1748,7 @@ std::vector<tc::Tile> stage1_tiles(const BatchPlan& pl, int nt) {
 }
 
 void plan_splits(BatchPlan& pl, cudaStream_t s) {
+  std::vector<SplitArgs> jobs;
   for (size_t i = 0; i < pl.probs.size(); ++i) {
     const bse_problem& p = pl.probs[i].p;
     const int n = (int)pl.probs[i].n;
@@ -1717,13 +1756,13 @@ void plan_splits(BatchPlan& pl, cudaStream_t s) {
                  pl.Kp, n, pl.pieces, 1, p.v_bar, pl.xa.as<__nv_bfloat16>(), pl.x_rows,
                  pl.x_row0[i]};
     sa.c64 = p.in_dtype == BSE_C64;
-    launch_split(sa, s);
+    jobs.push_back(sa);
     SplitArgs sb = sa;
     sb.conj = 0;
     sb.kscale = nullptr;
     sb.out = pl.xb.as<__nv_bfloat16>();
     sb.bneg = 1;
-    launch_split(sb, s);
+    jobs.push_back(sb);
   }
   for (BatchPlan::Term& t : pl.terms) {
     const bse_problem& p = pl.probs[t.prob].p;
@@ -1734,13 +1773,13 @@ void plan_splits(BatchPlan& pl, cudaStream_t s) {
                  t.w_row0};
     sw.bneg = 1;
     sw.c64 = p.in_dtype == BSE_C64;
-    if (t.w_owner) launch_split(sw, s);
+    if (t.w_owner) jobs.push_back(sw);
     SplitArgs sa{reinterpret_cast<const double2*>(t.side), SPLIT_PAIRS, t.perm.as<int>(),
                  t.rows_side, 0, pl.ng, pl.Kp, npair * t.rows_side, pl.pieces, 0, nullptr,
                  pl.asplit.as<__nv_bfloat16>(), pl.a_rows, t.a_row0};
     sa.pair_nb = t.side_nb;
     sa.c64 = p.in_dtype == BSE_C64;
-    launch_split(sa, s);
+    jobs.push_back(sa);
     if (t.tc2) {   // the other pair side, in pair order, conjugated as opX
       SplitArgs sx{t.s2.x, SPLIT_PAIRS, t.x2perm.as<int>(), t.s2.rows_x, 0, pl.ng, pl.Kp,
                    npair * t.s2.rows_x, pl.pieces, t.s2.conj_x, nullptr,
@@ -1749,9 +1788,10 @@ void plan_splits(BatchPlan& pl, cudaStream_t s) {
       sx.pair_nb = t.x_nb;
       sx.bneg = t.rows_t_side ? 1 : 0;   // the B operand when T forms the tile rows
       sx.c64 = p.in_dtype == BSE_C64;
-      launch_split(sx, s);
+      jobs.push_back(sx);
     }
   }
+  launch_splits(jobs, s);
 }
 
 // blocks k > k' of A and B from their mirrors, for the problems whose
@@ -2777,12 +2817,80 @@ __global__ void k_rpa_reduce(const float2* part, int splits, int64_t nn, double2
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nn;
        i += (int64_t)gridDim.x * blockDim.x) {
     double sx = 0.0, sy = 0.0;
+#pragma unroll 8
     for (int s = 0; s < splits; ++s) {
       const float2 p = part[(int64_t)s * nn + i];
-      sx += (double)p.x;
-      sy += (double)p.y;
+      sx += f32_to_f64_bits(p.x);   // (conversions would double the FP64 work)
+      sy += f32_to_f64_bits(p.y);
     }
     x[i] = make_double2(sx, sy);
+  }
+}
+
+// Both operands of the RPA product from one read of the pair elements: rows G,
+// K = transitions a, element m[a][G] f[a] (FP32 scale), split; A the conjugate.
+// Tiles of 32 G x 64 transitions through shared memory, so that reads (along G)
+// and writes (along a) are contiguous: bound by HBM (25,600 transitions, NG =
+// 500: 115 us; two passes with strided plane stores took 370 us).
+struct RpaSplitArgs {
+  const double2* m;
+  const double* f;
+  int64_t ntr, kp;
+  int ng;
+  __nv_bfloat16 *a, *b;   // [2P][ng][kp], [3P][ng][kp]
+};
+template <int P>
+__global__ void __launch_bounds__(256) k_rpa_split(RpaSplitArgs a) {
+  __shared__ uint32_t re[64][33], im[64][33];
+  const int64_t k0 = (int64_t)blockIdx.x * 64;
+  const int g0 = blockIdx.y * 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint4* src = reinterpret_cast<const uint4*>(a.m);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int kl = warp + 8 * i;
+    const int64_t k = k0 + kl;
+    uint32_t fr = 0u, fi = 0u;
+    if (k < a.ntr && g0 + lane < a.ng) {
+      const uint4 x = __ldg(src + k * a.ng + g0 + lane);
+      const float sc = (float)a.f[k];
+      fr = __float_as_uint(__uint_as_float(f64w_to_f32_bits(x.x, x.y)) * sc);
+      fi = __float_as_uint(__uint_as_float(f64w_to_f32_bits(x.z, x.w)) * sc);
+    }
+    re[kl][lane] = fr;
+    im[kl][lane] = fi;
+  }
+  __syncthreads();
+  const int g = threadIdx.x >> 3, kq = (threadIdx.x & 7) * 8;
+  if (g0 + g >= a.ng) return;   // (kp is a multiple of 64: every k of the tile is a column)
+  uint32_t hr[P][8], hi[P][8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    uint32_t tr[P], ti[P];
+    split_f32_bf16<P>(re[kq + e][g], tr);
+    split_f32_bf16<P>(im[kq + e][g], ti);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      hr[p][e] = tr[p];
+      hi[p][e] = ti[p];
+    }
+  }
+  const int64_t plane = (int64_t)a.ng * a.kp, o = (int64_t)(g0 + g) * a.kp + k0 + kq;
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    uint4 vr, vi;
+    vr.x = hr[p][0] | (hr[p][1] << 16); vr.y = hr[p][2] | (hr[p][3] << 16);
+    vr.z = hr[p][4] | (hr[p][5] << 16); vr.w = hr[p][6] | (hr[p][7] << 16);
+    vi.x = hi[p][0] | (hi[p][1] << 16); vi.y = hi[p][2] | (hi[p][3] << 16);
+    vi.z = hi[p][4] | (hi[p][5] << 16); vi.w = hi[p][6] | (hi[p][7] << 16);
+    const uint4 vn = make_uint4(vi.x ^ 0x80008000u, vi.y ^ 0x80008000u, vi.z ^ 0x80008000u,
+                                vi.w ^ 0x80008000u);
+    // the pieces of -x are the negated pieces of x (rounding to nearest is symmetric)
+    *reinterpret_cast<uint4*>(a.a + (int64_t)p * plane + o) = vr;
+    *reinterpret_cast<uint4*>(a.a + (int64_t)(P + p) * plane + o) = vn;
+    *reinterpret_cast<uint4*>(a.b + (int64_t)(3 * p) * plane + o) = vn;
+    *reinterpret_cast<uint4*>(a.b + (int64_t)(3 * p + 1) * plane + o) = vr;
+    *reinterpret_cast<uint4*>(a.b + (int64_t)(3 * p + 2) * plane + o) = vi;
   }
 }
 }  // namespace
@@ -2797,29 +2905,27 @@ void rpa_x_mixed(int nk, int nv, int nc, int ng, const double* e_v, const double
   const int splits = (int)(kp / kspan);
   const int nt = tile_cols(round_up(ng, 32), kspan);
   const tc::GemmShape sh = make_shape(nt, kspan, pieces);
-  DevMem f((size_t)ntr * sizeof(double));
-  DevMem ap((size_t)tc::a_planes(pieces) * ng * kp * 2);
-  DevMem bp((size_t)tc::b_planes(pieces) * ng * kp * 2);
-  DevMem part((size_t)splits * ng * ng * sizeof(float2));
-  DevMem err(2 * sizeof(int));
-  BSE_CUDA(cudaMemsetAsync(err.ptr, 0, sizeof(int), s));
+  // stream-ordered workspace: hundreds of MB of cudaMalloc and cudaFree per call
+  // took longer than the product
+  DeviceBuffer f((size_t)ntr * sizeof(double), s);
+  DeviceBuffer ap((size_t)tc::a_planes(pieces) * ng * kp * 2, s);
+  DeviceBuffer bp((size_t)tc::b_planes(pieces) * ng * kp * 2, s);
+  DeviceBuffer part((size_t)splits * ng * ng * sizeof(float2), s);
+  DeviceBuffer err(2 * sizeof(int), s);
+  BSE_CUDA(cudaMemsetAsync(err.ptr, 0, 2 * sizeof(int), s));
   {
     Phase ph("rpa_split", s);
     k_rpa_inv_sqrt_gap<<<(int)std::min<int64_t>((ntr + 255) / 256, 152 * 8), 256, 0, s>>>(
         ntr, nv, nc, e_v, e_c_kq, f.as<double>());
+    const RpaSplitArgs sa{reinterpret_cast<const double2*>(m), f.as<double>(), ntr, kp, ng,
+                          ap.as<__nv_bfloat16>(), bp.as<__nv_bfloat16>()};
+    const dim3 grid((unsigned)(kp / 64), (unsigned)((ng + 31) / 32));
+    if (pieces == 3)
+      k_rpa_split<3><<<grid, 256, 0, s>>>(sa);
+    else
+      k_rpa_split<2><<<grid, 256, 0, s>>>(sa);
     BSE_CUDA(cudaGetLastError());
-    note_launches(1);
-    // rows G, K = transitions: element (G, a) is m[a][G] (transposed read)
-    SplitArgs sa{reinterpret_cast<const double2*>(m), SPLIT_DENSE, nullptr, 0, 0, (int)ntr,
-                 (int)kp, ng, pieces, 1, f.as<double>(), ap.as<__nv_bfloat16>(), ng, 0};
-    sa.tdense = 1;
-    sa.src_ld = ng;
-    launch_split(sa, s);
-    SplitArgs sb = sa;
-    sb.conj = 0;
-    sb.bneg = 1;
-    sb.out = bp.as<__nv_bfloat16>();
-    launch_split(sb, s);
+    note_launches(2);
   }
   std::vector<tc::Tile> tiles;
   for (int sp = 0; sp < splits; ++sp)
@@ -2827,7 +2933,9 @@ void rpa_x_mixed(int nk, int nv, int nc, int ng, const double* e_v, const double
       for (int n0 = 0; n0 < ng; n0 += nt)
         tiles.push_back({m0, std::min(tc::BM, ng - m0), n0, n0, std::min(nt, ng - n0), m0, sp,
                          sp * RPA_KSTEPS});
-  DevMem dtiles = upload_mem(tiles);
+  DeviceBuffer dtiles(tiles.size() * sizeof(tc::Tile), s);
+  BSE_CUDA(cudaMemcpyAsync(dtiles.ptr, tiles.data(), tiles.size() * sizeof(tc::Tile),
+                           cudaMemcpyHostToDevice, s));
   const CUtensorMap ma = make_plane_map(ap.as<__nv_bfloat16>(), (int)kp, ng, tc::a_planes(pieces),
                                         tc::BM);
   const CUtensorMap mb = make_plane_map(bp.as<__nv_bfloat16>(), (int)kp, ng, tc::b_planes(pieces),
