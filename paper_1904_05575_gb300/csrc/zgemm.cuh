@@ -88,22 +88,49 @@ zgemm_batched(Prob P, int b0) {
     }
 }
 
+// The tile that leaves the fewest outputs (padding included) on the busiest SM:
+// the FP64 pipe (1.8 FMAs per clock and SM) bounds every tile, operand loads
+// none (a 16 x 16 tile loads 1 byte per clock), so what counts is padding and an
+// even spread.  432 x 432 x 181 took 785 us as 49 tiles of 64 x 64 (the pipe's
+// time on all SMs is 240), 729 blocks of 16 x 16 x 181 took 988 us in tiles of
+// 16 x 64; 264 and 266 us by this rule.  Every tile adds over k in
+// the same order: the same bits.
+struct ZTile {
+  int tm, tn;
+};
+inline ZTile zgemm_tile(int M, int N, int64_t batch, int sms) {
+  ZTile best{64, 64};
+  double least = 0.0;
+  for (const ZTile t : {ZTile{64, 64}, ZTile{32, 32}, ZTile{16, 64}, ZTile{16, 16}}) {
+    const int64_t blocks = (int64_t)((M + t.tm - 1) / t.tm) * ((N + t.tn - 1) / t.tn) * batch;
+    // outputs on the busiest SM; a smaller tile has to gain a twentieth
+    const double load = (double)((blocks + sms - 1) / sms) * t.tm * t.tn;
+    if (least == 0.0 || load < 0.95 * least) {
+      least = load;
+      best = t;
+    }
+  }
+  return best;
+}
+
 template <class Prob>
 void launch_zgemm(const Prob& P, int batch, cudaStream_t s) {
-  // tile shape from the output shape; every config is 128 or 256 threads.
+  int dev = 0, sms = 152;
+  BSE_CUDA(cudaGetDevice(&dev));
+  BSE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const ZTile t = zgemm_tile(P.M, P.N, batch, sms);
   // gridDim.z is capped at 65535, so large batches go in chunks.
   for (int b0 = 0; b0 < batch; b0 += 65535) {
     const int nb = batch - b0 < 65535 ? batch - b0 : 65535;
-    if (P.M >= 48 && P.N >= 48) {
-      dim3 grid((P.N + 63) / 64, (P.M + 63) / 64, nb);
+    const dim3 grid((P.N + t.tn - 1) / t.tn, (P.M + t.tm - 1) / t.tm, nb);
+    if (t.tm == 64)
       zgemm_batched<64, 64, 8, 4, 4, Prob><<<grid, 256, 0, s>>>(P, b0);
-    } else if (P.M <= 16) {
-      dim3 grid((P.N + 63) / 64, (P.M + 15) / 16, nb);
-      zgemm_batched<16, 64, 16, 2, 4, Prob><<<grid, 128, 0, s>>>(P, b0);
-    } else {
-      dim3 grid((P.N + 31) / 32, (P.M + 31) / 32, nb);
+    else if (t.tm == 32)
       zgemm_batched<32, 32, 16, 2, 4, Prob><<<grid, 128, 0, s>>>(P, b0);
-    }
+    else if (t.tn == 64)
+      zgemm_batched<16, 64, 16, 2, 4, Prob><<<grid, 128, 0, s>>>(P, b0);
+    else
+      zgemm_batched<16, 16, 16, 1, 2, Prob><<<grid, 128, 0, s>>>(P, b0);
     BSE_CUDA(cudaGetLastError());
     note_launches(1);
   }
