@@ -140,6 +140,12 @@ void davidson_fp64(int n, const bse_c128* A, const bse_c128* B, int64_t ld, int 
                    int matvec_precision = BSE_PREC_FP64, const bse_c128* V0 = nullptr,
                    int k0 = 0);
 
+// The k lowest eigenpairs of a small Hermitian matrix (eig_small.cu): work of
+// eig_lowest_workspace(m) bytes (device); false: not served (S untouched).
+size_t eig_lowest_workspace(int m);
+bool eig_lowest(int m, double2* S, int lds, int k, double* lam, void* work, cudaStream_t s);
+bool tridiagonal_lowest(int m, const double* d, const double* e, int k, double* lam, double* Z);
+
 // Hermitian matrix-vector blocks on the tensor cores (build_mixed.cu): A and
 // B split once; apply writes AV = A V and BV = B V (n x k, column-major, ld n).
 // Nothing here waits for the device except tc_matvec_check, which throws

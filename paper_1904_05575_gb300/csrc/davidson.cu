@@ -17,7 +17,7 @@
 // Gram-Schmidt passes by GEMM, then Cholesky QR twice) and appended; the
 // basis restarts from the current Ritz vectors when full.
 // Small dense steps (projections, m x m factorisations) are cuBLAS / cuSOLVER
-// calls; the host drives the iteration and reads residual norms each step.
+// calls, the projected eigenproblem is eig_small.cu's; the host drives the iteration and reads residual norms each step.
 #include <cublas_v2.h>
 #include <cuda_runtime.h>
 #include <cusolverDn.h>
@@ -162,7 +162,7 @@ struct Solver {
   LibHandles h;
   DeviceBuffer V, P, M, AV, BV, ap, am, L, S, U, W, R1, R2, T, C, info, dE, dF, dD, dDp, dDm,
       dS;
-  std::unique_ptr<DeviceBuffer> work_;
+  std::unique_ptr<DeviceBuffer> work_, eig_;
   int lwork = 0;
   int m = 0;          // current basis size
   int m_proj = 0;     // columns of the projected a+ and a- already computed
@@ -199,6 +199,7 @@ struct Solver {
                                              &lw2));
     lwork = std::max(std::max(lw1, lw2), 1);
     work_.reset(new DeviceBuffer((size_t)lwork * 16, s));
+    eig_.reset(new DeviceBuffer(eig_lowest_workspace(mmax), s));
   }
 
   cuDoubleComplex* col(const DeviceBuffer& b, int j, int64_t ldb) const {
@@ -364,14 +365,18 @@ struct Solver {
     BSE_CUBLAS(cublasZtrmm(h.blas, CUBLAS_SIDE_LEFT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_C,
                            CUBLAS_DIAG_NON_UNIT, m, m, &one, L.as<cuDoubleComplex>(), mmax,
                            W.as<cuDoubleComplex>(), mmax, S.as<cuDoubleComplex>(), mmax));
-    BSE_CUSOLVER(cusolverDnZheevd(h.solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_LOWER, m,
-                                  S.as<cuDoubleComplex>(), mmax, dE.as<double>(),
-                                  work_->as<cuDoubleComplex>(), lwork, info.as<int>()));
+    // the k lowest pairs; the library's full eigensolve where eig_lowest does not
+    // serve (m > 512, or pairs it could not separate)
     std::vector<double> e2(m);
-    BSE_CUDA(cudaMemcpyAsync(e2.data(), dE.ptr, m * 8, cudaMemcpyDeviceToHost, s));
-    BSE_CUDA(cudaMemcpyAsync(&hinfo, info.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BSE_CUDA(cudaStreamSynchronize(s));
-    if (hinfo != 0) throw Error(BSE_ERR_CUDA, "zheevd on the projected problem failed");
+    if (!eig_lowest(m, S.as<double2>(), mmax, k, e2.data(), eig_->ptr, s)) {
+      BSE_CUSOLVER(cusolverDnZheevd(h.solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_LOWER, m,
+                                    S.as<cuDoubleComplex>(), mmax, dE.as<double>(),
+                                    work_->as<cuDoubleComplex>(), lwork, info.as<int>()));
+      BSE_CUDA(cudaMemcpyAsync(e2.data(), dE.ptr, m * 8, cudaMemcpyDeviceToHost, s));
+      BSE_CUDA(cudaMemcpyAsync(&hinfo, info.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
+      BSE_CUDA(cudaStreamSynchronize(s));
+      if (hinfo != 0) throw Error(BSE_ERR_CUDA, "zheevd on the projected problem failed");
+    }
     E.assign(k, 0.0);
     std::vector<double> f(k);
     for (int j = 0; j < k; ++j) {
