@@ -2627,6 +2627,10 @@ __global__ void __launch_bounds__(256) k_matvec_reduce(int n, int ncols, int nse
   out[o] = y;
 }
 
+// Planes up to this size (one matrix, N = 9,450) come from the stream-ordered
+// pool, which keeps them for the next call; larger ones go back to the device
+// when the object goes.
+constexpr size_t kMatvecPoolBytes = 1ull << 30;
 constexpr size_t kMatvecPartBytes = (size_t)512 << 20;   // most scratch for split-K partial sums
 }  // namespace
 
@@ -2645,6 +2649,8 @@ struct TcMatvec {
   const bse_c128* A = nullptr;   // caller's A (its diagonal, in FP64)
   int64_t ld = 0;
   std::unique_ptr<DeviceBuffer> ap, bp, vp, part, err;
+  DevMem ap_large, bp_large;     // planes above kMatvecPoolBytes
+  __nv_bfloat16 *a_planes = nullptr, *b_planes = nullptr;
   struct TileList {
     std::vector<tc::Tile> host;            // kept until the copy has been read
     std::unique_ptr<DeviceBuffer> dev;
@@ -2698,8 +2704,13 @@ TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t 
   m->split_cols = (int)std::max<size_t>(1, std::min<size_t>(kmax, kMatvecPartBytes / col_bytes));
   m->part.reset(new DeviceBuffer(m->split_cols * col_bytes, s));
   const size_t mat_bytes = (size_t)m->planes * n * m->Kp * 2;
-  m->ap.reset(new DeviceBuffer(mat_bytes, s));
-  if (B) m->bp.reset(new DeviceBuffer(mat_bytes, s));
+  auto planes_of = [&](std::unique_ptr<DeviceBuffer>& pooled, DevMem& large) {
+    if (mat_bytes > kMatvecPoolBytes) large = DevMem(mat_bytes);
+    else pooled.reset(new DeviceBuffer(mat_bytes, s));
+    return static_cast<__nv_bfloat16*>(large.ptr ? large.ptr : pooled->ptr);
+  };
+  m->a_planes = planes_of(m->ap, m->ap_large);
+  if (B) m->b_planes = planes_of(m->bp, m->bp_large);
   const size_t v_bytes = (size_t)tc::b_planes(m->pieces) * m->kmax_rows * m->Kp * 2;
   m->vp.reset(new DeviceBuffer(v_bytes, s));
   BSE_CUDA(cudaMemsetAsync(m->vp->ptr, 0, v_bytes, s));
@@ -2708,13 +2719,13 @@ TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t 
   for (int which = 0; which < (B ? 2 : 1); ++which) {
     SplitArgs sa{reinterpret_cast<const double2*>(which ? B : A), SPLIT_DENSE, nullptr, 0, 0, n,
                  m->Kp, n, m->pieces, 1, nullptr,
-                 (which ? m->bp : m->ap)->as<__nv_bfloat16>(), n, 0};
+                 which ? m->b_planes : m->a_planes, n, 0};
     sa.src_ld = ld;
     sa.zero_diag = which == 0;
     launch_split(sa, s);
   }
-  m->ma_a = make_plane_map(m->ap->as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
-  if (B) m->ma_b = make_plane_map(m->bp->as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
+  m->ma_a = make_plane_map(m->a_planes, m->Kp, n, m->planes, tc::BM);
+  if (B) m->ma_b = make_plane_map(m->b_planes, m->Kp, n, m->planes, tc::BM);
   m->mb_v = make_plane_map(m->vp->as<__nv_bfloat16>(), m->Kp, m->kmax_rows,
                            tc::b_planes(m->pieces), m->nt);
   matvec_tiles(m.get(), 1, true, s);   // uploaded here: later products may be captured
