@@ -154,6 +154,69 @@ __global__ void k_gather_cols(int n, int k, const int* idx, const double2* x, do
     y[i + (int64_t)j * n] = x[i + (int64_t)idx[j] * n];
 }
 
+// part[b] = V(rows b kc ..)^H Y(rows b kc ..): one K range of C = V^H Y per batch
+struct VhyProb {
+  int M, N, K;          // K = kc
+  const double2 *V, *Y;
+  int64_t ldv, ldy;
+  int rows;             // length of the columns of V and Y
+  double2* part;        // [batch][N][M]
+  __device__ cplx a(int b, int m, int k) const {
+    const int64_t r = (int64_t)b * K + k;
+    if (r >= rows) return {0.0, 0.0};
+    const double2 v = V[(int64_t)m * ldv + r];
+    return {v.x, -v.y};
+  }
+  __device__ cplx b(int b, int n, int k) const {
+    const int64_t r = (int64_t)b * K + k;
+    if (r >= rows) return {0.0, 0.0};
+    const double2 v = Y[(int64_t)n * ldy + r];
+    return {v.x, v.y};
+  }
+  __device__ void store(int b, int m, int n, cplx v) const {
+    part[((int64_t)b * N + n) * M + m] = make_double2(v.x, v.y);
+  }
+};
+__global__ void k_vhy_sum(int M, int N, int batches, const double2* part, double2* C, int64_t ldc) {
+  const int64_t mn = (int64_t)M * N;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < mn;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    double2 t = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int b = 0; b < batches; ++b) {
+      const double2 p = part[b * mn + i];
+      t.x += p.x;
+      t.y += p.y;
+    }
+    C[i % M + i / M * ldc] = t;
+  }
+}
+// C = beta C + alpha V G (columns of V combined)
+struct VgProb {
+  int M, N, K;
+  const double2 *V, *G;
+  int64_t ldv, ldg, ldc;
+  double alpha, beta;
+  double2* C;
+  __device__ cplx a(int, int m, int k) const {
+    const double2 v = V[(int64_t)k * ldv + m];
+    return {v.x, v.y};
+  }
+  __device__ cplx b(int, int n, int k) const {
+    const double2 v = G[(int64_t)n * ldg + k];
+    return {v.x, v.y};
+  }
+  __device__ void store(int, int m, int n, cplx v) const {
+    double2* c = C + (int64_t)n * ldc + m;
+    double2 o = make_double2(alpha * v.x, alpha * v.y);
+    if (beta != 0.0) {
+      o.x = fma(beta, c->x, o.x);
+      o.y = fma(beta, c->y, o.y);
+    }
+    *c = o;
+  }
+};
+
 struct Solver {
   int n, nev, mmax;
   const bse_c128 *A, *B;
@@ -206,6 +269,59 @@ struct Solver {
     return b.as<cuDoubleComplex>() + (int64_t)j * ldb;
   }
 
+  // The tall-skinny products of an iteration.  Their outputs make few library
+  // tiles (V^H Y of 192 x 16 is three of 64 x 32, each running over all n rows
+  // on one SM at 1.8 FP64 FMAs per clock), so below two 64 x 64 tiles per SM
+  // they run on the FP64 GEMM kernel with tiles that spread over the GPU, V^H Y
+  // in ranges of K whose sums are added in order; from there on the library's
+  // tiles fill the GPU.  Rank 2,560, 8 excitons, 24 iterations: appending to
+  // the basis 34.8 -> 16.3 ms, residuals 10.7 -> 8.0 ms, projections and W
+  // 63.5 -> 58.1 ms against the library; the whole call 97 -> 72.5 ms.
+  static bool skinny(int64_t M, int64_t N) { return ((M + 63) / 64) * ((N + 63) / 64) < 2 * 152; }
+  std::unique_ptr<DeviceBuffer> part_;
+  size_t part_bytes = 0;
+
+  // C = V^H Y, V: n x M, Y: n x N (leading dimension n)
+  void vhy(const cuDoubleComplex* Vp, int M, const cuDoubleComplex* Y, int N, cuDoubleComplex* C,
+           int ldc) {
+    if (!skinny(M, N)) {
+      const cuDoubleComplex one = make_cuDoubleComplex(1, 0), zero = make_cuDoubleComplex(0, 0);
+      BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, M, N, n, &one, Vp, n, Y, n, &zero, C,
+                             ldc));
+      return;
+    }
+    // about four 16 x 16 tiles per SM over all ranges, ranges of at least 64 rows
+    const int tiles = ((M + 15) / 16) * ((N + 15) / 16);
+    int batches = std::max(1, std::min((n + 63) / 64, 4 * 152 / tiles));
+    const int kc = ((n + batches - 1) / batches + 15) / 16 * 16;
+    batches = (n + kc - 1) / kc;
+    const size_t need = (size_t)batches * M * N * 16;
+    if (need > part_bytes) {
+      part_.reset(new DeviceBuffer(need, s));
+      part_bytes = need;
+    }
+    VhyProb p{M, N, kc, reinterpret_cast<const double2*>(Vp), reinterpret_cast<const double2*>(Y), n, n,
+              n, part_->as<double2>()};
+    launch_zgemm(p, batches, s);
+    k_vhy_sum<<<(int)std::min<int64_t>(((int64_t)M * N + 127) / 128, 152 * 8), 128, 0, s>>>(
+        M, N, batches, part_->as<double2>(), reinterpret_cast<double2*>(C), ldc);
+    BSE_CUDA(cudaGetLastError());
+    note_launches(1);
+  }
+  // C = beta C + alpha V G, V: rows x K, G: K x N
+  void vg(int rows, const cuDoubleComplex* Vp, int ldv, const cuDoubleComplex* Gp, int ldg, int N, int K,
+          cuDoubleComplex* C, int ldc, double alpha, double beta) {
+    if (!skinny(rows, N)) {
+      const cuDoubleComplex al = make_cuDoubleComplex(alpha, 0), be = make_cuDoubleComplex(beta, 0);
+      BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, rows, N, K, &al, Vp, ldv, Gp, ldg, &be, C,
+                             ldc));
+      return;
+    }
+    VgProb p{rows, N, K, reinterpret_cast<const double2*>(Vp), reinterpret_cast<const double2*>(Gp),
+             ldv, ldg, ldc, alpha, beta, reinterpret_cast<double2*>(C)};
+    launch_zgemm(p, 1, s);
+  }
+
   // tensor-core matvecs (split-precision A, B), or NULL for the FP64 kernel
   TcMatvec* tcm = nullptr;
 
@@ -243,8 +359,7 @@ struct Solver {
   // working precision.  Returns the number appended.
   int append_block(cuDoubleComplex* X, int b) {
     if (b <= 0 || m >= mmax) return 0;
-    const cuDoubleComplex one = make_cuDoubleComplex(1, 0), zero = make_cuDoubleComplex(0, 0),
-                          mone = make_cuDoubleComplex(-1, 0);
+    const cuDoubleComplex one = make_cuDoubleComplex(1, 0), zero = make_cuDoubleComplex(0, 0);
     std::vector<double> n0(b);
     k_col_norms<<<b, 256, 0, s>>>(n, reinterpret_cast<const double2*>(X), nullptr, n,
                                   nrm.as<double>());
@@ -253,15 +368,12 @@ struct Solver {
     BSE_CUDA(cudaMemcpyAsync(n0.data(), nrm.ptr, (size_t)b * 8, cudaMemcpyDeviceToHost, s));
     auto project = [&](cuDoubleComplex* Y, int k) {
       if (m == 0) return;
-      BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, m, k, n, &one,
-                             V.as<cuDoubleComplex>(), n, Y, n, &zero, G.as<cuDoubleComplex>(), m));
-      BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, k, m, &mone,
-                             V.as<cuDoubleComplex>(), n, G.as<cuDoubleComplex>(), m, &one, Y, n));
+      vhy(V.as<cuDoubleComplex>(), m, Y, k, G.as<cuDoubleComplex>(), m);
+      vg(n, V.as<cuDoubleComplex>(), n, G.as<cuDoubleComplex>(), m, k, m, Y, n, -1.0, 1.0);
     };
     // Gram matrix of k columns to the host (column-major k x k)
     auto gram = [&](const cuDoubleComplex* Y, int k, std::vector<cuDoubleComplex>& g) {
-      BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, k, k, n, &one, Y, n, Y, n, &zero,
-                             G.as<cuDoubleComplex>(), k));
+      vhy(Y, k, Y, k, G.as<cuDoubleComplex>(), k);
       g.resize((size_t)k * k);
       BSE_CUDA(cudaMemcpyAsync(g.data(), G.ptr, (size_t)k * k * 16, cudaMemcpyDeviceToHost, s));
       BSE_CUDA(cudaStreamSynchronize(s));
@@ -329,17 +441,13 @@ struct Solver {
 
   // projected problem on the current basis; fills U (u, m x nev), W (w, m x nev), E (host)
   void rayleigh_ritz(int k, std::vector<double>& E) {
-    const cuDoubleComplex one = make_cuDoubleComplex(1, 0), zero = make_cuDoubleComplex(0, 0);
+    const cuDoubleComplex one = make_cuDoubleComplex(1, 0);
     // a+ = V^H P, a- = V^H M: only the columns of the vectors added since the
     // last step (the basis only grows between restarts); the rows of the new
     // vectors in the old columns follow from Hermiticity
     const int m0 = m_proj < m ? m_proj : 0, nw = m - m0;
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, m, nw, n, &one,
-                           V.as<cuDoubleComplex>(), n, P.as<cuDoubleComplex>() + (int64_t)m0 * n, n,
-                           &zero, ap.as<cuDoubleComplex>() + (int64_t)m0 * mmax, mmax));
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_C, CUBLAS_OP_N, m, nw, n, &one,
-                           V.as<cuDoubleComplex>(), n, M.as<cuDoubleComplex>() + (int64_t)m0 * n, n,
-                           &zero, am.as<cuDoubleComplex>() + (int64_t)m0 * mmax, mmax));
+    vhy(V.as<cuDoubleComplex>(), m, col(P, m0, n), nw, col(ap, m0, mmax), mmax);
+    vhy(V.as<cuDoubleComplex>(), m, col(M, m0, n), nw, col(am, m0, mmax), mmax);
     m_proj = m;
     dim3 tb(16, 16), gb((m + 15) / 16, (m + 15) / 16);
     dim3 gn((m + 15) / 16, (nw + 15) / 16);
@@ -392,9 +500,8 @@ struct Solver {
     k_scale_cols<<<dim3((m + 127) / 128, k), 128, 0, s>>>(m, k, U.as<double2>(), mmax,
                                                           dF.as<double>());
     // w = a+ u / E
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, m, k, m, &one,
-                           ap.as<cuDoubleComplex>(), mmax, U.as<cuDoubleComplex>(), mmax, &zero,
-                           W.as<cuDoubleComplex>(), mmax));
+    vg(m, ap.as<cuDoubleComplex>(), mmax, U.as<cuDoubleComplex>(), mmax, k, m, W.as<cuDoubleComplex>(),
+       mmax, 1.0, 0.0);
     for (int j = 0; j < k; ++j) f[j] = 1.0 / E[j];
     BSE_CUDA(cudaMemcpyAsync(dF.ptr, f.data(), k * 8, cudaMemcpyHostToDevice, s));
     k_scale_cols<<<dim3((m + 127) / 128, k), 128, 0, s>>>(m, k, W.as<double2>(), mmax,
@@ -405,28 +512,21 @@ struct Solver {
 
   // r+ = P u - V (w E), r- = M w - V (u E) into R1, R2 (n x k); returns max column norms
   void residuals(int k, const std::vector<double>& E, std::vector<double>& res) {
-    const cuDoubleComplex one = make_cuDoubleComplex(1, 0), zero = make_cuDoubleComplex(0, 0),
-                          mone = make_cuDoubleComplex(-1, 0);
     // X+Y and X-Y as full vectors, scaled by E: T[:, 0:k] = V (w E), T[:, k:2k] = V (u E)
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, k, m, &one,
-                           V.as<cuDoubleComplex>(), n, W.as<cuDoubleComplex>(), mmax, &zero,
-                           T.as<cuDoubleComplex>(), n));
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, k, m, &one,
-                           V.as<cuDoubleComplex>(), n, U.as<cuDoubleComplex>(), mmax, &zero,
-                           col(T, k, n), n));
+    cuDoubleComplex *t0 = T.as<cuDoubleComplex>(), *t1 = col(T, k, n);
+    vg(n, V.as<cuDoubleComplex>(), n, W.as<cuDoubleComplex>(), mmax, k, m, t0, n, 1.0, 0.0);
+    vg(n, V.as<cuDoubleComplex>(), n, U.as<cuDoubleComplex>(), mmax, k, m, t1, n, 1.0, 0.0);
     k_scale_cols<<<dim3((n + 127) / 128, k), 128, 0, s>>>(n, k, T.as<double2>(), n, dE.as<double>());
     k_scale_cols<<<dim3((n + 127) / 128, k), 128, 0, s>>>(n, k, T.as<double2>() + (int64_t)k * n, n,
                                                           dE.as<double>());
     note_launches(2);
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, k, m, &one,
-                           P.as<cuDoubleComplex>(), n, U.as<cuDoubleComplex>(), mmax, &zero,
-                           R1.as<cuDoubleComplex>(), n));
-    BSE_CUBLAS(cublasZaxpy(h.blas, n * k, &mone, T.as<cuDoubleComplex>(), 1,
-                           R1.as<cuDoubleComplex>(), 1));
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, k, m, &one,
-                           M.as<cuDoubleComplex>(), n, W.as<cuDoubleComplex>(), mmax, &zero,
-                           R2.as<cuDoubleComplex>(), n));
-    BSE_CUBLAS(cublasZaxpy(h.blas, n * k, &mone, col(T, k, n), 1, R2.as<cuDoubleComplex>(), 1));
+    // R1 = P u - T0, R2 = M w - T1
+    BSE_CUDA(cudaMemcpyAsync(R1.ptr, t0, (size_t)n * k * 16, cudaMemcpyDeviceToDevice, s));
+    BSE_CUDA(cudaMemcpyAsync(R2.ptr, t1, (size_t)n * k * 16, cudaMemcpyDeviceToDevice, s));
+    vg(n, P.as<cuDoubleComplex>(), n, U.as<cuDoubleComplex>(), mmax, k, m, R1.as<cuDoubleComplex>(), n,
+       1.0, -1.0);
+    vg(n, M.as<cuDoubleComplex>(), n, W.as<cuDoubleComplex>(), mmax, k, m, R2.as<cuDoubleComplex>(), n,
+       1.0, -1.0);
     res.assign(k, 0.0);
     k_col_norms<<<k, 256, 0, s>>>(n, R1.as<double2>(), R2.as<double2>(), n, nrm.as<double>());
     BSE_CUDA(cudaGetLastError());
@@ -670,14 +770,11 @@ void davidson_fp64(int n, const bse_c128* A, const bse_c128* B, int64_t ld, int 
     // restart from the Ritz vectors when the new block would not fit
     Phase ph_o("davidson_basis", s);
     if (sv.m + 2 * nt > mmax) {
-      const cuDoubleComplex one = make_cuDoubleComplex(1, 0), zero = make_cuDoubleComplex(0, 0);
       // X+Y and X-Y of the kr lowest pairs into R1 (n x 2 kr), then rebuild V
-      BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, kr, sv.m, &one,
-                             sv.V.as<cuDoubleComplex>(), n, sv.U.as<cuDoubleComplex>(), mmax,
-                             &zero, sv.R1.as<cuDoubleComplex>(), n));
-      BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, kr, sv.m, &one,
-                             sv.V.as<cuDoubleComplex>(), n, sv.W.as<cuDoubleComplex>(), mmax,
-                             &zero, sv.R1.as<cuDoubleComplex>() + (int64_t)kr * n, n));
+      sv.vg(n, sv.V.as<cuDoubleComplex>(), n, sv.U.as<cuDoubleComplex>(), mmax, kr, sv.m,
+            sv.R1.as<cuDoubleComplex>(), n, 1.0, 0.0);
+      sv.vg(n, sv.V.as<cuDoubleComplex>(), n, sv.W.as<cuDoubleComplex>(), mmax, kr, sv.m,
+            sv.col(sv.R1, kr, n), n, 1.0, 0.0);
       sv.m = 0;
       sv.m_proj = 0;
       sv.append_block(sv.R1.as<cuDoubleComplex>(), 2 * kr);
@@ -692,12 +789,9 @@ void davidson_fp64(int n, const bse_c128* A, const bse_c128* B, int64_t ld, int 
 
   // outputs: E and X+Y = V u for the nev lowest
   BSE_CUDA(cudaMemcpyAsync(E_out, E.data(), (size_t)k * 8, cudaMemcpyHostToDevice, s));
-  if (XpY_out) {
-    const cuDoubleComplex one = make_cuDoubleComplex(1, 0), zero = make_cuDoubleComplex(0, 0);
-    BSE_CUBLAS(cublasZgemm(h.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, k, sv.m, &one,
-                           sv.V.as<cuDoubleComplex>(), n, sv.U.as<cuDoubleComplex>(), mmax, &zero,
-                           reinterpret_cast<cuDoubleComplex*>(XpY_out), n));
-  }
+  if (XpY_out)
+    sv.vg(n, sv.V.as<cuDoubleComplex>(), n, sv.U.as<cuDoubleComplex>(), mmax, k, sv.m,
+          reinterpret_cast<cuDoubleComplex*>(XpY_out), n, 1.0, 0.0);
   BSE_CUDA(cudaStreamSynchronize(s));
   if (!converged)
     throw Error(BSE_ERR_NO_CONV, "Davidson did not reach the residual tolerance in " +
