@@ -16,8 +16,10 @@
 // trained MLP of mlp.cu), orthogonalised against V as one block (two
 // Gram-Schmidt passes by GEMM, then Cholesky QR twice) and appended; the
 // basis restarts from the current Ritz vectors when full.
-// Small dense steps (projections, m x m factorisations) are cuBLAS / cuSOLVER
-// calls, the projected eigenproblem is eig_small.cu's; the host drives the iteration and reads residual norms each step.
+// The tall-skinny products run on the FP64 GEMM kernel, the projected
+// eigenproblem is eig_small.cu's; the m x m factorisations and triangular
+// products are cuBLAS / cuSOLVER calls.  The host drives the iteration and
+// reads residual norms each step.
 #include <cublas_v2.h>
 #include <cuda_runtime.h>
 #include <cusolverDn.h>

@@ -17,7 +17,8 @@
 // back on the library where it fails or m is too large.  Bound by the latency
 // of the reduction's chain per column (two grid exchanges, a square root, two
 // divisions and three block sums, about 7 us): the projected problems of that
-// solve take 2.6 instead of 6.4 ms per iteration, the solve 95 instead of 166.
+// solve take 2.6 instead of 6.4 ms per iteration, the solve 97 instead of 166
+// (72.5 with the tall-skinny products of davidson.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>

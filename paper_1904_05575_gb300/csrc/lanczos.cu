@@ -295,15 +295,14 @@ __device__ __forceinline__ void split_into_planes(const TcMatvecIo& io, int i, d
 }
 
 // out = the product of v: its K segments' partial sums added in segment order
-// (FP32) plus the FP64 diagonal term; coef[slot] += Re(conj(v) out).  32 rows
-// per block: eight warps stage the segments in shared memory (all loads in
+// (FP32) plus the FP64 diagonal term; wsum[block] = the block's part of
+// Re(conj(v) out).  32 rows per block: eight warps stage the segments in shared memory (all loads in
 // flight at once), then one warp adds them in order; one thread per row
 // walking the segments itself took 13 us at N = 4,860 (38 dependent rounds on
 // 19 blocks).
 constexpr int kRedSegs = 64;   // segments staged at a time
 __global__ void __launch_bounds__(256) k_tc_reduce_dot(int n, TcMatvecIo io, const double2* v,
-                                                       double2* out, double* coef,
-                                                       const int* jbase, int slot) {
+                                                       double2* out, double* wsum) {
   __shared__ float2 st[kRedSegs][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * 32 + lane;
@@ -340,16 +339,50 @@ __global__ void __launch_bounds__(256) k_tc_reduce_dot(int n, TcMatvecIo io, con
     d = w.x * o.x + w.y * o.y;
   }
   for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-  if (lane == 0) atomicAdd(coef + (jbase ? 2 * *jbase : 0) + slot, d);
+  if (lane == 0) wsum[blockIdx.x] = d;
 }
 
-// y_{j+1} (unnormalised) = u - alpha_j y_j - beta_{j-1} y_{j-1}, split for the next product
-__global__ void k_tc_y(int n, TcMatvecIo io, const double2* u, const double2* y, const double2* yprev,
-                       const double* coef, const int* jbase, int q, double2* ynew) {
+// The dot product from its per-block parts, in every thread of a block of 128:
+// groups of eight parts (256 rows) by a tree, the groups in order.  One order,
+// so that a run repeats bit for bit (with atomic additions eps changed by up to
+// 1e-9 from run to run: the recursion amplifies the last bits).
+__device__ __forceinline__ double tc_dot(const double* wsum, int parts) {
+  __shared__ double gs[128];
+  __shared__ double total;
+  double acc = 0.0;
+  const int groups = (parts + 7) / 8;
+  for (int g0 = 0; g0 < groups; g0 += 128) {
+    const int g = g0 + threadIdx.x;
+    if (g < groups) {
+      double w[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) w[q] = 8 * g + q < parts ? __ldg(wsum + 8 * g + q) : 0.0;
+      gs[threadIdx.x] = ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int q = 0; q < min(128, groups - g0); ++q) acc += gs[q];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) total = acc;
+  __syncthreads();
+  return total;
+}
+__global__ void __launch_bounds__(128) k_tc_total(const double* wsum, int parts, double* out) {
+  const double t = tc_dot(wsum, parts);
+  if (threadIdx.x == 0) *out = t;
+}
+
+// alpha_j and y_{j+1} (unnormalised) = u - alpha_j y_j - beta_{j-1} y_{j-1}, split for the
+// next product
+__global__ void __launch_bounds__(128) k_tc_y(int n, TcMatvecIo io, const double2* u, const double2* y,
+                                              const double2* yprev, const double* wsum, int parts,
+                                              double* coef, const int* jbase, int q, double2* ynew) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
   const int j = *jbase + q;
-  const double a = coef[2 * j];
+  const double a = tc_dot(wsum, parts);
+  if (i == 0) coef[2 * j] = a;
+  if (i >= n) return;
   const double b = j > 0 ? sqrt(fmax(coef[2 * j - 1], 0.0)) : 0.0;
   const double2 uy = u[i], y1 = y[i], y0 = yprev[i];
   const double2 o = make_double2(uy.x - a * y1.x - b * y0.x, uy.y - a * y1.y - b * y0.y);
@@ -357,15 +390,17 @@ __global__ void k_tc_y(int n, TcMatvecIo io, const double2* u, const double2* y,
   split_into_planes(io, i, o);
 }
 
-// v = x / beta, y_prev <- y <- y_new / beta (beta^2 = coef[slot], slot 2j - 1
-// before step j), v split for the next product
-__global__ void k_tc_scale(int n, TcMatvecIo io, const double* coef, const int* jbase, int q,
-                           int nv2_slot, const double2* x, double2* v, const double2* ynew,
-                           double2* y, double2* yprev) {
+// beta_{j-1}^2 (<v_0, v_0> before step 0) and v = x / beta, y_prev <- y <- y_new / beta, v
+// split for the next product
+__global__ void __launch_bounds__(128) k_tc_scale(int n, TcMatvecIo io, const double* wsum, int parts,
+                                                  double* coef, const int* jbase, int q,
+                                                  const double2* x, double2* v, const double2* ynew,
+                                                  double2* y, double2* yprev) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
   const int j = *jbase + q;
-  const double b2 = coef[j > 0 ? 2 * j - 1 : nv2_slot];
+  const double b2 = tc_dot(wsum, parts);
+  if (i == 0 && j > 0) coef[2 * j - 1] = b2;
+  if (i >= n) return;
   const double f = b2 > 0.0 ? 1.0 / sqrt(b2) : 0.0;
   const double2 xv = x[i], yv = ynew[i];
   const double2 o = make_double2(xv.x * f, xv.y * f);
@@ -474,7 +509,7 @@ __global__ void __launch_bounds__(256) k_eps_change(int n_omega, const double2* 
 // a CUDA graph and replayed (the step index lives on the device, the vectors
 // stay in place), so that no launch waits for the host and the products are
 // bound by reading the 12 N^2 bytes of planes.  A step at N = 4,860 takes
-// 137 us; it took 430 us when each product uploaded its tile list and
+// 140 us; it took 430 us when each product uploaded its tile list and
 // synchronised and ran on 38 blocks (one per 128 rows, all of K each).
 int spectrum_lanczos(int n, const bse_c128* A, const bse_c128* B, int64_t ld, const bse_c128* rho,
                      double c_q, double vc, int n_omega, const double* omega, double delta,
@@ -492,7 +527,8 @@ int spectrum_lanczos(int n, const bse_c128* A, const bse_c128* B, int64_t ld, co
   DeviceBuffer bv(tc ? vb : 0, s), bx(vb, s), by0(vb, s), by1(vb, s), by2(vb, s), bu(vb, s),
       coef((size_t)ncoef * sizeof(double), s),
       ea((size_t)std::max(n_omega, 1) * sizeof(double2), s), diff(2 * sizeof(double), s),
-      ctl(4 * sizeof(int), s), part((size_t)2 * kLzMaxBlocks * sizeof(double), s);
+      ctl(4 * sizeof(int), s), part((size_t)2 * kLzMaxBlocks * sizeof(double), s),
+      dots(tc ? (size_t)((n + 31) / 32) * sizeof(double) : 0, s);
   double* cf = coef.as<double>();
   int* ct = ctl.as<int>();   // [0] first step of the captured graph; [2], [3] grid exchange
   const int eb = (n + 127) / 128, rb = (n + 31) / 32;
@@ -554,13 +590,14 @@ int spectrum_lanczos(int n, const bse_c128* A, const bse_c128* B, int64_t ld, co
   // one tensor-core step (place q of a captured graph) on stream st
   double2 *V = bv.as<double2>(), *X = bx.as<double2>(), *U = bu.as<double2>(),
           *Y = by0.as<double2>(), *Yp = by1.as<double2>(), *Yn = by2.as<double2>();
+  double* ws = dots.as<double>();
   auto tc_step = [&](cudaStream_t st, int q) {
-    k_tc_scale<<<eb, 128, 0, st>>>(n, iop, cf, ct, q, nv2_slot, X, V, Yn, Y, Yp);
-    tc_matvec_products(mp, st);                                             // u = (A+B) v_j
-    k_tc_reduce_dot<<<rb, 256, 0, st>>>(n, iop, V, U, cf, ct, 2 * q);       // alpha_j
-    k_tc_y<<<eb, 128, 0, st>>>(n, iod, U, Y, Yp, cf, ct, q, Yn);
-    tc_matvec_products(md, st);                                             // x = (A-B) y
-    k_tc_reduce_dot<<<rb, 256, 0, st>>>(n, iod, Yn, X, cf, ct, 2 * q + 1);  // beta_j^2
+    k_tc_scale<<<eb, 128, 0, st>>>(n, iop, ws, rb, cf, ct, q, X, V, Yn, Y, Yp);
+    tc_matvec_products(mp, st);                                  // u = (A+B) v_j
+    k_tc_reduce_dot<<<rb, 256, 0, st>>>(n, iop, V, U, ws);       // alpha_j
+    k_tc_y<<<eb, 128, 0, st>>>(n, iod, U, Y, Yp, ws, rb, cf, ct, q, Yn);
+    tc_matvec_products(md, st);                                  // x = (A-B) y
+    k_tc_reduce_dot<<<rb, 256, 0, st>>>(n, iod, Yn, X, ws);      // beta_j^2
     BSE_CUDA(cudaGetLastError());
   };
   auto step_add = [&](cudaStream_t st, int by) { k_step_add<<<1, 1, 0, st>>>(ct, by); };
@@ -581,8 +618,9 @@ int spectrum_lanczos(int n, const bse_c128* A, const bse_c128* B, int64_t ld, co
   if (tc) {
     BSE_CUDA(cudaMemsetAsync(Y, 0, vb, s));   // becomes y_{-1}
     tc_matvec_products(md, s);
-    k_tc_reduce_dot<<<rb, 256, 0, s>>>(n, iod, Yn, X, cf, nullptr, nv2_slot);
-    launches += 1;
+    k_tc_reduce_dot<<<rb, 256, 0, s>>>(n, iod, Yn, X, ws);
+    k_tc_total<<<1, 128, 0, s>>>(ws, rb, cf + nv2_slot);
+    launches += 2;
   } else {
     fp64_steps(0, 0);
   }

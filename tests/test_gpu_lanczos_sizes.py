@@ -66,3 +66,18 @@ def test_lanczos_sizes(bse, n, prec, with_b):
     ref = _eps_closed(e, w, rho, omega, 0.05, 4 * np.pi, 100.0 * n)
     bound = 1e-7 if prec == 0 else 1e-5
     assert np.abs(eps.cpu().numpy() - ref).max() < bound * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n,prec", [(31, 2), (257, 2), (2100, 2), (1025, 0)])
+def test_lanczos_repeats_bit_for_bit(bse, n, prec):
+    import torch
+    e, w, rho = _case(n)
+    wt = torch.as_tensor(w).cuda()
+    A = wt.conj()[:, None] * wt[None, :]
+    A.diagonal().add_(torch.as_tensor(e).cuda())
+    omega = torch.linspace(0.0, 10.0, 301, dtype=torch.float64, device="cuda")
+    eps = [torch.empty(301, dtype=torch.complex128, device="cuda") for _ in range(3)]
+    for x in eps:
+        bse.bse_spectrum_lanczos(n, A, torch.zeros_like(A), torch.as_tensor(rho).cuda(), 4 * np.pi,
+                                 100.0 * n, omega, 0.05, x, tol=1e-10, matvec_precision=prec)
+    assert torch.equal(eps[0], eps[1]) and torch.equal(eps[0], eps[2])
