@@ -306,8 +306,9 @@ int bse_spectrum(int32_t n, bse_c128* S_inout, const bse_c128* L, int64_t ld,
  * products by A+B and A-B per step and no factorisation, gives Q as a
  * continued fraction of its coefficients.  The steps stop when eps changes
  * by at most tol times max |eps| between checks (every 48 steps with FP64
- * products, which run as a CUDA graph of 6 steps, every 50 with tensor-core
- * products; fewer for n < 50; at least min(100, 2n) steps); steps_out
+ * products, which run as one cooperative launch, every 50 with tensor-core
+ * products, which run as a CUDA graph of 10 steps; fewer for n < 50; at least
+ * min(100, 2n) steps); steps_out
  * (host, may be NULL) receives the number.
  * A, B as for bse_reduce (B = NULL: zero), rho, omega, delta, c_q, vc as for
  * bse_spectrum (delta > 0); eps_out [n_omega] device.  A+B and A-B are
@@ -315,10 +316,12 @@ int bse_spectrum(int32_t n, bse_c128* S_inout, const bse_c128* L, int64_t ld,
  * BSE_PREC_FP64 (products in FP64 on CUDA cores) or BSE_PREC_BF16X6 /
  * BF16X3 (A+B and A-B split once into BF16 pieces, products on the tensor
  * cores with the diagonal in FP64, as for bse_lowest_excitons; a further
- * 2 x 12 N^2 bytes for BF16X6); the recursion itself is FP64.
+ * 2 x 12 N^2 bytes for BF16X6 and 16 N bytes per 128 columns of partial
+ * sums); the recursion itself is FP64.
  * Syncs at each check.  Errors: BSE_ERR_ARG, BSE_ERR_NOT_PD
  * (conj(rho)^H (A-B) conj(rho) <= 0), BSE_ERR_NO_CONV (max_steps reached;
- * eps_out holds the last estimate), BSE_ERR_NOMEM, BSE_ERR_CUDA. */
+ * eps_out holds the last estimate), BSE_ERR_NOMEM, BSE_ERR_CUDA,
+ * BSE_ERR_TIMEOUT (a bounded wait of a kernel expired). */
 int bse_spectrum_lanczos(int32_t n, const bse_c128* A, const bse_c128* B, int64_t ld,
                          const bse_c128* rho, double c_q, double vc, int32_t n_omega,
                          const double* omega, double delta, double tol, int32_t max_steps,
@@ -359,9 +362,11 @@ int bse_spectrum_tensor(int32_t n, const bse_c128* Z, const bse_c128* L, int64_t
  * transitions, BSE_PREC_BF16X6 / BF16X3 the tensor cores (the transitions
  * split into BF16 pieces, FP32 accumulation over ranges of 512 transitions);
  * the partial sums are added in FP64.  eps and w are formed in FP64, eps^-1
- * by cuSOLVER LU.  Syncs.  Errors: BSE_ERR_ARG (sizes, NULL, a non-positive
+ * by Gauss-Jordan elimination of the Hermitian positive definite form
+ * V^-1 + 2 kappa X, V = diag(v) (cuSOLVER's pivoted LU of eps when a v_G is
+ * negative, a pivot fails or ng is above what shared memory holds).  Syncs.  Errors: BSE_ERR_ARG (sizes, NULL, a non-positive
  * gap, unknown precision), BSE_ERR_NOMEM, BSE_ERR_CUDA (also a singular eps),
- * BSE_ERR_TIMEOUT (a bounded wait of the tensor-core GEMM expired). */
+ * BSE_ERR_TIMEOUT (a bounded wait of a kernel expired). */
 int bse_rpa_screening(int32_t nk, int32_t nv, int32_t nc, int32_t ng, double omega_cell,
                       const double* e_v, const double* e_c_kq, const bse_c128* m, const double* v,
                       int32_t precision, bse_c128* w_out, void* cuda_stream);
@@ -435,14 +440,16 @@ int bse_xpy(int32_t n, int32_t k, const bse_c128* Z, const bse_c128* L, int64_t 
  *   matvec_precision  BSE_PREC_FP64: matvecs (A+B)V, (A-B)V by the FP64 GEMM;
  *              BSE_PREC_BF16X6 / BF16X3: A and B split once into BF16 pieces
  *              and the matvecs run on the tensor cores (FP32 accumulation in
- *              K segments, FP64 results); workspace 2 x 12 N^2 bytes (BF16X6).
+ *              K segments, FP64 results); workspace 2 x 12 N^2 bytes (BF16X6)
+ *              and up to 512 MiB of partial sums.
  *              The residual floor then scales with ~1e-7 of the off-diagonal
  *              part of A (A's diagonal is applied in FP64): keep tol_ev above it.
  *   E_out      [nev] device, ascending exciton energies (eV)
  *   XpY_out    [n x nev] device column-major, X+Y with (X+Y)^H (X-Y) = 1, or NULL
  *   iters_out  host, iterations used (may be NULL)
  * Syncs every iteration.  Errors: BSE_ERR_ARG, BSE_ERR_NOT_PD, BSE_ERR_NO_CONV
- * (E_out then holds the last estimates), BSE_ERR_UNSUPPORTED, BSE_ERR_CUDA. */
+ * (E_out then holds the last estimates), BSE_ERR_UNSUPPORTED, BSE_ERR_CUDA,
+ * BSE_ERR_TIMEOUT (a bounded wait of a kernel expired). */
 int bse_lowest_excitons(int32_t n, const bse_c128* A, const bse_c128* B, int64_t ld, int32_t nev,
                         double tol_ev, int32_t max_iter, int32_t precond, const void* mlp,
                         int32_t matvec_precision, double* E_out, bse_c128* XpY_out,
