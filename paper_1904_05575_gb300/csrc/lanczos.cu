@@ -126,6 +126,7 @@ __device__ __forceinline__ bool lz_exchange(const LzArgs& a, LzSmem& sm, int pha
       }
     }
   }
+  __syncwarp();   // lane 0's acquire orders the other lanes' reads below (a shuffle orders no memory)
   ok = __shfl_sync(0xffffffffu, ok, 0);
   if (!ok) return false;
   double p[kLzMaxBlocks / 32];
