@@ -223,6 +223,13 @@ int bse_plan_status(void* plan, void* cuda_stream);
  * the following executes.  FP64 plans have no bounded waits.  Errors:
  * BSE_ERR_ARG. */
 int bse_plan_set_wait_limit(void* plan, double seconds);
+/* The same budget (default about 2 s) for the calls of this host thread that take no
+ * plan and return BSE_ERR_TIMEOUT where a wait runs longer:
+ * bse_spectrum_lanczos, bse_lowest_excitons[_from], bse_mlp_trajectory_samples
+ * and bse_rpa_screening, also their FP64 forms (a wait is then one for the other
+ * blocks of a launch).  Outputs are incomplete after such an error; the next
+ * call starts afresh.  seconds in (0, 60].  Errors: BSE_ERR_ARG. */
+int bse_set_wait_limit(double seconds);
 /* output-column tile width the plan's stage-1 GEMM uses (0 for FP64 plans) */
 int bse_plan_tile_cols(const void* plan);
 /* The tensor-core stage-2 launches' output-column tile width and pipeline

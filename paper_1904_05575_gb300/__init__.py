@@ -68,7 +68,7 @@ EXPORTED = ("bse_build_kernel", "bse_reduce", "bse_spectrum", "bse_last_error", 
             "bse_plan_stage2_shape", "bse_spectrum_lanczos",
             "bse_plan_fused", "bse_spectrum_tensor", "bse_loss_function",
             "bse_lowest_excitons_from", "bse_rpa_screening", "bse_plan_set_wait_limit",
-            "bse_pair_elements")
+            "bse_pair_elements", "bse_set_wait_limit")
 
 
 def load(path: str = LIB_PATH) -> ctypes.CDLL:
@@ -120,6 +120,8 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.bse_pair_elements.argtypes = [i32, i32, i32, i32, i32, vp, vp, vp, vp, i32, i32, vp, vp,
                                       vp, vp, vp]
     lib.bse_pair_elements.restype = ctypes.c_int
+    lib.bse_set_wait_limit.argtypes = [dbl]
+    lib.bse_set_wait_limit.restype = ctypes.c_int
     lib.bse_plan_set_wait_limit.restype = ctypes.c_int
     for name in ("bse_plan_create", "bse_plan_execute", "bse_plan_status", "bse_plan_tile_cols",
                  "bse_plan_fused"):
@@ -454,6 +456,11 @@ def bse_pair_elements(grid: int, cv, cc, basis, gout, m_x=None, m_vv=None, m_cc=
         b.ctypes.data_as(ctypes.c_void_p), g.ctypes.data_as(ctypes.c_void_p), int(k_begin),
         int(k_count), ptr(m_x, "m_x"), ptr(m_vv, "m_vv"), ptr(m_cc, "m_cc"), ptr(n_vc, "n_vc"),
         _stream(stream)))
+
+
+def bse_set_wait_limit(seconds: float) -> None:
+    """Clock budget of the bounded device waits in this thread's calls without a plan."""
+    _check(load().bse_set_wait_limit(float(seconds)))
 
 
 def bse_phase_timing(enable: bool) -> None:

@@ -26,7 +26,15 @@ void set_last_error(const std::string& msg) { g_last_error = msg; }
 
 namespace {
 std::atomic<int64_t> g_launches{0};
+thread_local long long t_wait = kDefaultWaitCycles;   // bse_set_wait_limit
+}  // namespace
+long long wait_cycles(double seconds) {
+  int dev = 0, khz = 0;
+  BSE_CUDA(cudaGetDevice(&dev));
+  BSE_CUDA(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev));
+  return std::max<long long>(1, (long long)(seconds * 1e3 * (khz > 0 ? khz : 2000000)));
 }
+long long call_wait_cycles() { return t_wait; }
 void note_launches(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 namespace {
@@ -348,6 +356,13 @@ extern "C" int bse_plan_stage2_shape(const void* plan, int32_t* tile_cols, int32
 
 extern "C" int bse_plan_fused(const void* plan) {
   return plan ? plan_fused(static_cast<const BatchPlan*>(plan)) : 0;
+}
+
+extern "C" int bse_set_wait_limit(double seconds) {
+  return guarded([&] {
+    BSE_CHECK_ARG(seconds > 0.0 && seconds <= 60.0, "wait limit must be in (0, 60] seconds");
+    t_wait = wait_cycles(seconds);
+  });
 }
 
 extern "C" int bse_plan_set_wait_limit(void* plan, double seconds) {

@@ -29,6 +29,12 @@ void set_last_error(const std::string& msg);
 // Count of kernels launched by this library (see bse_kernel_launches).
 void note_launches(int64_t n);
 
+// Clock budget of a bounded device wait: the default (about 2 s), of `seconds` on the current device, and
+// of the calls this host thread makes without a plan (bse_set_wait_limit).
+constexpr long long kDefaultWaitCycles = 4000000000LL;
+long long wait_cycles(double seconds);
+long long call_wait_cycles();
+
 // RAII phase timer: when bse_phase_timing(1) is on, records a start event on
 // construction and a stop event on destruction, both on the given stream.
 class Phase {

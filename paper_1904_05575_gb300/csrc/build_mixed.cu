@@ -2446,10 +2446,7 @@ void plan_stage2_shape(const BatchPlan* pl, int* tile_cols, int* stages) {
 int plan_fused(const BatchPlan* pl) { return pl->fused ? 1 : 0; }
 
 void plan_set_wait(BatchPlan* pl, double seconds) {
-  int khz = 0;
-  BSE_CUDA(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, pl->device));
-  const double cycles = seconds * 1e3 * (khz > 0 ? khz : 2000000);
-  pl->wait = std::max<long long>(1, (long long)cycles);
+  pl->wait = wait_cycles(seconds);
 }
 
 void plan_destroy(BatchPlan* pl) { delete pl; }
@@ -2690,6 +2687,7 @@ TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t 
   m->kmax_rows = single ? 8 : round_up(kmax, 32);
   m->nt = single ? 8 : tile_cols(m->kmax_rows, m->Kp);
   m->sh = make_shape(m->nt, m->Kp, m->pieces);
+  m->sh.wait = call_wait_cycles();
   // the segments of the whole-K form (see mma_role); the last one may run past
   // the padded K, where the planes read as zero
   m->seg_len = (m->sh.kchunks + m->sh.ksegs - 1) / m->sh.ksegs;
@@ -2915,7 +2913,8 @@ void rpa_x_mixed(int nk, int nv, int nc, int ng, const double* e_v, const double
   if (kp > INT32_MAX) throw Error(BSE_ERR_UNSUPPORTED, "too many transitions for the RPA GEMM");
   const int splits = (int)(kp / kspan);
   const int nt = tile_cols(round_up(ng, 32), kspan);
-  const tc::GemmShape sh = make_shape(nt, kspan, pieces);
+  tc::GemmShape sh = make_shape(nt, kspan, pieces);
+  sh.wait = call_wait_cycles();
   // stream-ordered workspace: hundreds of MB of cudaMalloc and cudaFree per call
   // took longer than the product
   DeviceBuffer f((size_t)ntr * sizeof(double), s);

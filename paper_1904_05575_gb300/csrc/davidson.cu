@@ -479,6 +479,7 @@ struct Solver {
     // serve (m > 512, or pairs it could not separate)
     std::vector<double> e2(m);
     if (!eig_lowest(m, S.as<double2>(), mmax, k, e2.data(), eig_->ptr, s)) {
+      Phase ph("davidson_zheevd", s);
       BSE_CUSOLVER(cusolverDnZheevd(h.solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_LOWER, m,
                                     S.as<cuDoubleComplex>(), mmax, dE.as<double>(),
                                     work_->as<cuDoubleComplex>(), lwork, info.as<int>()));

@@ -33,7 +33,6 @@ namespace {
 
 constexpr int kTrdThreads = 256, kTrdBlocks = 64, kTrdMaxM = 512;
 constexpr int kTrdMaxK = 64;   // (orthogonalising k close vectors costs k^2 m on the host)
-constexpr long long kTrdWait = 4000000000LL;   // clock budget of a grid barrier (~2 s)
 
 struct TrdArgs {
   int m, lds;
@@ -42,6 +41,7 @@ struct TrdArgs {
   double *d, *e;
   double2 *col, *p;     // [2][m] exchange buffers
   int *arrived, *gave_up;
+  long long wait;       // clock budget of a grid barrier
 };
 
 __device__ __forceinline__ bool trd_barrier(const TrdArgs& a, int target, int* ok_s) {
@@ -54,14 +54,13 @@ __device__ __forceinline__ bool trd_barrier(const TrdArgs& a, int target, int* o
       int seen;
       asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(a.arrived) : "memory");
       if (seen >= target) break;
-      if ((spin & 63) == 0) {
-        int stop;
+      int stop = clock64() - t0 > a.wait;
+      if (!stop && (spin & 63) == 0)
         asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(stop) : "l"(a.gave_up) : "memory");
-        if (stop || clock64() - t0 > kTrdWait) {
-          atomicExch(a.gave_up, 1);
-          ok = 0;
-          break;
-        }
+      if (stop) {
+        atomicExch(a.gave_up, 1);
+        ok = 0;
+        break;
       }
     }
     *ok_s = ok;
@@ -403,7 +402,7 @@ bool eig_lowest(int m, double2* S, int lds, int k, double* lam, void* work, cuda
   const int blocks = std::min(kTrdBlocks, m), rows = (m + blocks - 1) / blocks;
   const size_t smem = ((size_t)rows + 2) * m * sizeof(double2);
   BSE_CUDA(cudaFuncSetAttribute(k_hetrd, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-  TrdArgs a{m, lds, S, V, tau, de, de + m, col, p, ctl, ctl + 1};
+  TrdArgs a{m, lds, S, V, tau, de, de + m, col, p, ctl, ctl + 1, call_wait_cycles()};
   void* args[] = {&a};
   BSE_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_hetrd), dim3(blocks),
                                        dim3(kTrdThreads), args, smem, s));

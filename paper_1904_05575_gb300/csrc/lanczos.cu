@@ -63,7 +63,6 @@ constexpr int kLzThreads = 512;          // 15 warps of products, 1 of scalars
 constexpr int kLzProd = kLzThreads - 32;
 constexpr int kLzCols = 1024;            // columns staged in shared memory at a time
 constexpr int kLzMaxBlocks = 160;
-constexpr long long kLzWait = 4000000000LL;   // clock budget of one exchange (~2 s)
 
 struct LzArgs {
   int n;
@@ -76,6 +75,7 @@ struct LzArgs {
   double* part;             // [2][kLzMaxBlocks] per-block partial sums (of even and odd exchanges)
   int* arrived;             // arrivals at the exchanges, zeroed before the launch
   int* gave_up;             // a bounded wait expired
+  long long wait;           // clock budget of one exchange
   int rows;                 // rows per block
   int j0, steps;            // first step, number of steps; steps = 0: x = (A-B) y[0] and <v, v> only
 };
@@ -115,14 +115,13 @@ __device__ __forceinline__ bool lz_exchange(const LzArgs& a, LzSmem& sm, int pha
       int seen;
       asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(a.arrived) : "memory");
       if (seen >= target) break;
-      if ((spin & 63) == 0) {
-        int stop;
+      int stop = clock64() - t0 > a.wait;
+      if (!stop && (spin & 63) == 0)
         asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(stop) : "l"(a.gave_up) : "memory");
-        if (stop || clock64() - t0 > kLzWait) {
-          atomicExch(a.gave_up, 1);
-          ok = 0;
-          break;
-        }
+      if (stop) {
+        atomicExch(a.gave_up, 1);
+        ok = 0;
+        break;
       }
     }
   }
@@ -578,7 +577,7 @@ int spectrum_lanczos(int n, const bse_c128* A, const bse_c128* B, int64_t ld, co
   const int blocks = (n + rows - 1) / rows;
   LzArgs lz{n, Cp, Dp, ldp, bx.as<double2>(), bu.as<double2>(),
             {by0.as<double2>(), by1.as<double2>(), by2.as<double2>()}, cf, nv2_slot,
-            part.as<double>(), ct + 2, ct + 3, rows, 0, 0};
+            part.as<double>(), ct + 2, ct + 3, call_wait_cycles(), rows, 0, 0};
   auto fp64_steps = [&](int j0, int steps) {
     lz.j0 = j0;
     lz.steps = steps;

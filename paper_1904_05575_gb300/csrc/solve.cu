@@ -542,7 +542,6 @@ __global__ void k_rpa_w(int ng, const double* v, const double2* inv, double2* w)
 // serial pivot blocks; 1.7 ms at NG = 500, where the pivoted LU and solve of the
 // library took about 6 ms.
 constexpr int kGjNb = 16, kGjThreads = 256, kGjMaxSmem = 160 * 1024;
-constexpr long long kGjWait = 4000000000LL;   // clock budget of a grid barrier (~2 s)
 
 struct GjArgs {
   int n, cols;            // matrix size, columns per block
@@ -551,6 +550,7 @@ struct GjArgs {
   double2* panel;         // [2][kGjNb][n] the columns being eliminated
   double2* w;             // row-major result v_G (eps^-1)_GG'
   int *arrived, *bad;     // zeroed; bad: 1 pivot, 2 a barrier gave up
+  long long wait;         // clock budget of a grid barrier
 };
 
 __device__ __forceinline__ bool gj_barrier(const GjArgs& a, int target, int* ok_s) {
@@ -563,14 +563,13 @@ __device__ __forceinline__ bool gj_barrier(const GjArgs& a, int target, int* ok_
       int seen;
       asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(a.arrived) : "memory");
       if (seen >= target) break;
-      if ((spin & 63) == 0) {
-        int stop;
+      int stop = clock64() - t0 > a.wait ? 2 : 0;
+      if (!stop && (spin & 63) == 0)
         asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(stop) : "l"(a.bad) : "memory");
-        if ((stop & 2) || clock64() - t0 > kGjWait) {
-          atomicOr(a.bad, 2);
-          ok = 0;
-          break;
-        }
+      if (stop & 2) {
+        atomicOr(a.bad, 2);
+        ok = 0;
+        break;
       }
     }
     *ok_s = ok;
@@ -707,7 +706,8 @@ bool gj_screening(int ng, const double2* eps, const double* v, double2* w, cudaS
                                 kGjMaxSmem));
   DeviceBuffer panel((size_t)2 * kGjNb * ng * sizeof(double2), s), ctl(2 * sizeof(int), s);
   BSE_CUDA(cudaMemsetAsync(ctl.ptr, 0, 2 * sizeof(int), s));
-  GjArgs a{ng, cols, eps, v, panel.as<double2>(), w, ctl.as<int>(), ctl.as<int>() + 1};
+  GjArgs a{ng, cols, eps, v, panel.as<double2>(), w, ctl.as<int>(), ctl.as<int>() + 1,
+           call_wait_cycles()};
   void* args[] = {&a};
   BSE_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_gj_screening), dim3(blocks),
                                        dim3(kGjThreads), args, smem, s));
@@ -762,6 +762,7 @@ void rpa_screening(int nk, int nv, int nc, int ng, double omega_cell, const doub
     note_launches(1);   // k_rpa_eps
     return;
   }
+  Phase ph("rpa_lu", s);
   // the row-major eps is, column-major, eps^T; its inverse (eps^T)^-1 =
   // (eps^-1)^T in column-major storage is eps^-1 in row-major storage
   int lwork = 0;

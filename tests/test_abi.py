@@ -155,3 +155,11 @@ def test_host_side_argument_errors_newer_entry_points(lib):
     q.m_x = 0x1004
     assert lib2.bse_build_kernel((bse.bse_problem * 1)(q), 1, 0, None) == bse.BSE_ERR_ARG
     assert b"8-byte" in lib2.bse_last_error()
+
+
+def test_wait_limit_range_is_checked_on_the_host():
+    import paper_1904_05575_gb300 as bse
+    lib2 = bse.load()
+    for bad in (0.0, -1.0, 60.5, float("nan"), float("inf")):
+        assert lib2.bse_set_wait_limit(bad) == bse.BSE_ERR_ARG
+    assert b"wait limit" in lib2.bse_last_error()
