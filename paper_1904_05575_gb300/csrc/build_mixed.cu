@@ -765,8 +765,7 @@ __global__ void __launch_bounds__(256) k_stage2_pipe(Stage2Args a) {
 // scheduler with ten warps per SM at 168 registers; the packed FMA pipe 44 %
 // busy).  4 x 12 bands, NG = 181, 4,096 pairs: W^rr (144 X rows, 16 T rows)
 // 1,453 -> 863 us, W^ra (48 x 48) 1,178 -> 735 us against 32 x 32 tiles with
-// 2 x 2 outputs per thread; 36 x 16 and 25 x 9 blocks (46,656 / 2 pairs, NG =
-// 113) 1,681 -> 1,491 us.  Tried and slower: 4 x 4 packed outputs per thread
+// 2 x 2 outputs per thread.  stage2_rows_pays says where it is used.  Tried and slower: 4 x 4 packed outputs per thread
 // with X converted through shared memory (861 / 803 us), fewer T rows per
 // thread for more warps (8: 1,159 / 1,043 us), 20 T rows for 40 x 40 blocks.
 constexpr int S2_GC = 8, S2_RING = 4, S2_MAXTH = 160, S2_MAXPB = 8;
@@ -1322,8 +1321,43 @@ struct S2Maps {   // k_stage2_rows: the tile and the tensor maps of its boxes
 
 // The kernel for the pair block (every variant adds in the same order: the
 // results do not depend on the choice).
-enum Stage2Form { S2F_SKINNY, S2F_MULTI, S2F_PIPE, S2F_24, S2F_40, S2F_ROWS };
-Stage2Form stage2_form(const Stage2Args& a) {
+enum Stage2Form { S2F_SKINNY, S2F_MULTI, S2F_PIPE, S2F_24, S2F_32X16, S2F_40X16, S2F_40, S2F_32, S2F_ROWS };
+Stage2Form stage2_tile_form(const Stage2Args& a, int64_t* outputs) {   // + outputs per pair, padding included
+  const int64_t x = a.rows_x, t = a.rows_t;
+  if (x <= 24 && t <= 24) return *outputs = 24 * 24, S2F_24;             // e.g. W^ra, 4 x 6 bands
+  if (x <= 32 && t <= 16) return *outputs = 32 * 16, S2F_32X16;          // e.g. W^rr, 3 x 5 bands (25 x 9)
+  if (x <= 40 && t <= 16) return *outputs = 40 * 16, S2F_40X16;          // e.g. W^rr, 4 x 6 bands (36 x 16)
+  if (x <= 40 && t <= 40) return *outputs = 40 * 40, S2F_40;             // e.g. W^ra, 2 x 20 bands (40 x 40)
+  return *outputs = (x + 31) / 32 * ((t + 31) / 32) * 32 * 32, S2F_32;
+}
+// The one-row form against the tiles: a tile form takes 0.37 ns per 1,000
+// outputs and plane wave once its blocks fill the GPU, the one-row form about
+// 1.15 times that, but it starts 18 us later at NG = 181 (28 against 10 us: two
+// to six warps per block, one ring of copies behind the other; 11 us at 91).  So
+// it takes the term where it computes a quarter fewer outputs and what it saves
+// on all pairs, saved = tile outputs - 1.15 row outputs, is worth that start:
+// 270,000 outputs by the figures, 500,000 here, so that no measured size loses.
+// NG = 181, us, tiles / one row: 48 x 48 with 108, 216, 729 and 4,096 pairs
+// (saved 1,446) 41 / 51, 72 / 65, 217 / 155, 1,143 / 735; 144 x 16 with 64, 216,
+// 4,096 (2,176) 39 / 67, 90 / 74, 1,407 / 863; 400 x 9 with 64, 108, 4,096
+// (6,688) 70 / 88, 111 / 82, 3,640 / 1,807; 25 x 9 with 729, 2,048, 15,625 (159)
+// 41 / 55, 96 / 96, 624 / 518.  Not a quarter fewer: 25 x 16 at 4,096 pairs
+// 174 / 264, 36 x 16 229 / 252.  Against several 32 x 32 tiles the one-row form
+// is also the faster one with as many outputs where plane waves and pairs are
+// many, by a few per cent: 4,096 pairs at NG = 181, both terms of 5 x 10 bands
+// (100 x 25, 50 x 50) 2,314 / 2,193, of 7 x 7 2,314 / 2,304; at NG = 91 1,243 /
+// 1,279 and 1,243 / 1,389, with 1,024 pairs 592 / 579 and 594 / 610.
+constexpr int64_t kS2RowsSaved = 500000;
+constexpr int kS2RowsManyNg = 160, kS2RowsManyPairs = 2000;
+bool stage2_rows_pays(const Stage2Args& a, int npair, int64_t tile_outputs) {
+  const S2Tile t = stage2_tile(a, npair);
+  const double rows = 2.0 * t.p * t.ntt * t.nxt * t.threads() / t.pb;
+  if (rows <= 0.75 * tile_outputs)
+    return npair * (tile_outputs - 1.15 * rows) >= (double)kS2RowsSaved;
+  return rows <= tile_outputs && tile_outputs > 40 * 40 && a.ng >= kS2RowsManyNg &&
+         npair >= kS2RowsManyPairs;
+}
+Stage2Form stage2_form(const Stage2Args& a, int npair) {
   // one X row per thread where T has at most 4 rows (bound by reading X once)
   if (stage2_skinny(a)) return S2F_SKINNY;
   // one output per thread where two whole blocks fit 256 threads that way, or one to 16 x 16
@@ -1331,16 +1365,16 @@ Stage2Form stage2_form(const Stage2Args& a) {
   if (a.rows_x <= 16 && a.rows_t <= 16) return S2F_PIPE;
   // nearly square blocks that one tile of 2 x 3 or 2 x 5 outputs per thread
   // covers: 24 x 24 (with 15 x 15 and 4 x 4: 1,231 us against 1,465 us for
-  // k_stage2_rows), 40 x 40 (755 against 974 us); with T rows for at most one
-  // k_stage2_rows tile that form is the faster one (36 x 16, 25 x 9)
-  if (a.rows_t > 16 && a.rows_x <= 24 && a.rows_t <= 24) return S2F_24;
-  if (a.rows_t > 24 && a.rows_x <= 40 && a.rows_t <= 40) return S2F_40;
-  return S2F_ROWS;
+  // k_stage2_rows), 40 x 40 (755 against 974 us)
+  int64_t outputs = 0;
+  const Stage2Form tiles = stage2_tile_form(a, &outputs);
+  if (tiles == S2F_24 || tiles == S2F_40) return tiles;
+  return stage2_rows_pays(a, npair, outputs) ? S2F_ROWS : tiles;
 }
 
 void launch_stage2(const Stage2Args& a, int npair, const S2Maps& m, int* err, long long wait,
                    cudaStream_t s) {
-  switch (stage2_form(a)) {
+  switch (stage2_form(a, npair)) {
     case S2F_SKINNY: {
       const int64_t total = (int64_t)npair * a.rows_x;
       const int64_t blocks = (total + SK_ROWS - 1) / SK_ROWS;
@@ -1354,7 +1388,10 @@ void launch_stage2(const Stage2Args& a, int npair, const S2Maps& m, int* err, lo
     }
     case S2F_PIPE: k_stage2_pipe<<<npair, 256, 0, s>>>(a); break;
     case S2F_24: launch_stage2_tiles<24, 24, 2, 3>(a, npair, s); break;
+    case S2F_32X16: launch_stage2_tiles<32, 16, 2, 2>(a, npair, s); break;
+    case S2F_40X16: launch_stage2_tiles<40, 16, 2, 2>(a, npair, s); break;
     case S2F_40: launch_stage2_tiles<40, 40, 2, 5>(a, npair, s); break;
+    case S2F_32: launch_stage2_tiles<32, 32, 2, 2>(a, npair, s); break;
     case S2F_ROWS: {
       const S2Tile& t = m.tile;
       const int64_t blocks = (int64_t)((npair + t.pb - 1) / t.pb) * t.nxt * t.ntt;
@@ -2303,7 +2340,7 @@ BatchPlan* plan_create(std::vector<Problem> probs, int precision, int flags, cud
       for (BatchPlan::Term& t : pl->terms) {
         t.s2.T = pl->tbuf.as<float2>();
         t.s2.t_ld = t_ld;
-        if (!t.tc2 && stage2_form(t.s2) == S2F_ROWS) {
+        if (!t.tc2 && stage2_form(t.s2, t.nact) == S2F_ROWS) {
           const Stage2Args& a = t.s2;
           const Problem& pr = pl->probs[t.prob];
           const int64_t x_pairs = a.x_transpose_pair ? (int64_t)pr.p.nk * pr.p.nk : pr.slab_pairs();
