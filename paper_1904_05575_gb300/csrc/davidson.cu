@@ -327,6 +327,15 @@ struct Solver {
   // tensor-core matvecs (split-precision A, B), or NULL for the FP64 kernel
   TcMatvec* tcm = nullptr;
 
+  // Waits for the stream; BSE_ERR_TIMEOUT if a wait expired in a product so far.
+  // Before anything is decided on P or M.
+  void sync_products() {
+    if (tcm)
+      tc_matvec_check(tcm, s);   // syncs
+    else
+      BSE_CUDA(cudaStreamSynchronize(s));
+  }
+
   // P, M for basis columns [j0, j1)
   void matvec(int j0, int j1) {
     const int k = j1 - j0;
@@ -463,7 +472,7 @@ struct Solver {
                                   mmax, work_->as<cuDoubleComplex>(), lwork, info.as<int>()));
     int hinfo = 0;
     BSE_CUDA(cudaMemcpyAsync(&hinfo, info.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BSE_CUDA(cudaStreamSynchronize(s));
+    sync_products();   // an expired wait comes before what its products say about the input
     if (hinfo != 0)
       throw Error(BSE_ERR_NOT_PD, "projected A-B is not positive definite (A-B or A+B not PD)");
     k_zero_strict_upper<<<gb, tb, 0, s>>>(m, L.as<double2>(), mmax);
@@ -535,10 +544,7 @@ struct Solver {
     BSE_CUDA(cudaGetLastError());
     note_launches(1);
     BSE_CUDA(cudaMemcpyAsync(res.data(), nrm.ptr, (size_t)k * 8, cudaMemcpyDeviceToHost, s));
-    if (tcm)
-      tc_matvec_check(tcm, s);   // syncs
-    else
-      BSE_CUDA(cudaStreamSynchronize(s));
+    BSE_CUDA(cudaStreamSynchronize(s));
   }
 };
 
@@ -656,6 +662,7 @@ void davidson_fp64(int n, const bse_c128* A, const bse_c128* B, int64_t ld, int 
     sv.append_block(sv.T.as<cuDoubleComplex>(), k0);
     sv.matvec(0, sv.m);
     m_done = sv.m;
+    sv.sync_products();
     BSE_CUDA(cudaMemcpyAsync(sv.T.ptr, sv.P.ptr, (size_t)n * m_done * 16, cudaMemcpyDeviceToDevice,
                              s));
     sv.append_block(sv.T.as<cuDoubleComplex>(), m_done);

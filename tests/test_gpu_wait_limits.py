@@ -130,3 +130,34 @@ def test_which_eigensolve_serves_the_projection(bse, nev, library):
 def test_which_inversion_serves_the_screening(bse, ng, library):
     """The unpivoted inversion while a block's columns fit shared memory, else LU."""
     assert ("rpa_lu" in _phases(bse, _screening(bse, ng, 0))) == library
+
+
+@pytest.mark.parametrize("warm", [False, True], ids=["cold", "warm"])
+def test_expired_product_is_a_timeout_not_a_statement_on_the_input(bse, warm):
+    """The products of a solve whose waits run out are whatever the workspace
+    held.  An earlier solve leaves a matrix there whose projection is not positive
+    definite; the next, of a positive definite matrix, must report the wait."""
+    import torch
+    n, k = 300, 4
+    good = _matrices(n)[0]
+    bad = torch.full((n, n), -10.0, dtype=torch.complex128, device="cuda")
+    bad.diagonal().copy_(torch.linspace(2.0, 6.0, n).cuda())
+    E = torch.empty(k, dtype=torch.float64, device="cuda")
+    start = torch.eye(n, dtype=torch.complex128, device="cuda")[:2 * k].contiguous() if warm else None
+
+    def call(A):
+        bse.bse_lowest_excitons(n, A, None, k, E, tol_ev=1e-5, max_iter=100, matvec_precision=2,
+                                start=start)
+
+    with pytest.raises(bse.BSEError) as err:
+        call(bad)
+    assert err.value.status == bse.BSE_ERR_NOT_PD
+    bse.bse_set_wait_limit(1e-9)
+    try:
+        with pytest.raises(bse.BSEError) as err:
+            call(good)
+    finally:
+        bse.bse_set_wait_limit(2.0)
+    assert err.value.status == bse.BSE_ERR_TIMEOUT
+    call(good)
+    assert torch.isfinite(E).all()
