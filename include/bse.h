@@ -369,10 +369,12 @@ int bse_spectrum_tensor(int32_t n, const bse_c128* Z, const bse_c128* L, int64_t
  * transitions, BSE_PREC_BF16X6 / BF16X3 the tensor cores (the transitions
  * split into BF16 pieces, FP32 accumulation over ranges of 512 transitions);
  * the partial sums are added in FP64.  eps and w are formed in FP64, eps^-1
- * by Gauss-Jordan elimination of the Hermitian positive definite form
- * V^-1 + 2 kappa X, V = diag(v) (cuSOLVER's pivoted LU of eps when a v_G is
- * negative, a pivot fails or ng is above what shared memory holds).  Syncs.  Errors: BSE_ERR_ARG (sizes, NULL, a non-positive
- * gap, unknown precision), BSE_ERR_NOMEM, BSE_ERR_CUDA (also a singular eps),
+ * by block Gauss-Jordan elimination of eps without pivoting: eps is similar,
+ * through V^1/2 where no v_G is zero, to 1 + 2 kappa V^1/2 X V^1/2, V = diag(v),
+ * whose pivots are >= 1.  cuSOLVER's pivoted LU of eps takes over when a v_G is
+ * negative, a pivot is below 1/2 (large v_G against the rounding of X) or ng is
+ * above what shared memory holds (about 1,200).  Syncs.  Errors: BSE_ERR_ARG
+ * (sizes, NULL, a non-positive gap, unknown precision), BSE_ERR_NOMEM, BSE_ERR_CUDA (also a singular eps),
  * BSE_ERR_TIMEOUT (a bounded wait of a kernel expired). */
 int bse_rpa_screening(int32_t nk, int32_t nv, int32_t nc, int32_t ng, double omega_cell,
                       const double* e_v, const double* e_c_kq, const bse_c128* m, const double* v,

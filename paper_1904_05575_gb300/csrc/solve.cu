@@ -532,8 +532,11 @@ __global__ void k_rpa_w(int ng, const double* v, const double2* inv, double2* w)
 // ---------------------------------------------------------------------------
 // eps = 1 + 2 kappa X diag(v) has the pivots of the Hermitian 1 + 2 kappa
 // v^1/2 X v^1/2 (a diagonal similarity), whose eigenvalues are >= 1 for v >= 0
-// and positive gaps: no pivoting is needed (an input with v < 0, a zero or a
-// non-finite pivot raises `bad` and the caller takes the pivoted LU).
+// and positive gaps, so that every pivot is >= 1: no pivoting is needed.  X has
+// the rounding of its products, though, and where 2 kappa v X times that reaches
+// one (BF16x3: about 1e-6 of X) the matrix need not be definite any more: a pivot
+// below 1/2 or not finite, or a v < 0, raises `bad` and the caller takes the
+// pivoted LU.
 // Each block owns a few columns and keeps them in shared memory from load to
 // result; a step eliminates kGjNb columns: the blocks that own them publish
 // them (double-buffered, one grid barrier per step), every block inverts the
@@ -612,7 +615,7 @@ __global__ void __launch_bounds__(kGjThreads, 1) k_gj_screening(GjArgs a) {
         const double2 d = D[p][p];
         const double q = 1.0 / fma(d.x, d.x, d.y * d.y);
         rp_s = make_double2(d.x * q, -d.y * q);
-        if (!(q > 0.0) || isinf(q)) bad = true;
+        if (!(d.x >= 0.5) || !(q > 0.0)) bad = true;
       }
       __syncthreads();
       const double2 rp = rp_s, prow = D[p][dc], pcol = D[dr][p], old = D[dr][dc];
