@@ -324,7 +324,7 @@ int bse_spectrum(int32_t n, bse_c128* S_inout, const bse_c128* L, int64_t ld,
  * BF16X3 (A+B and A-B split once into BF16 pieces, products on the tensor
  * cores with the diagonal in FP64, as for bse_lowest_excitons; a further
  * 2 x 12 N^2 bytes for BF16X6 and 16 N bytes per 128 columns of partial
- * sums); the recursion itself is FP64.
+ * sums, kept as there); the recursion itself is FP64.
  * Syncs at each check.  Errors: BSE_ERR_ARG, BSE_ERR_NOT_PD
  * (conj(rho)^H (A-B) conj(rho) <= 0), BSE_ERR_NO_CONV (max_steps reached;
  * eps_out holds the last estimate), BSE_ERR_NOMEM, BSE_ERR_CUDA,
@@ -368,7 +368,12 @@ int bse_spectrum_tensor(int32_t n, const bse_c128* Z, const bse_c128* L, int64_t
  * BSE_PREC_FP64 the FP64 GEMM kernel over ranges of at most 1,024
  * transitions, BSE_PREC_BF16X6 / BF16X3 the tensor cores (the transitions
  * split into BF16 pieces, FP32 accumulation over ranges of 512 transitions);
- * the partial sums are added in FP64.  eps and w are formed in FP64, eps^-1
+ * the partial sums are added in FP64.  Workspace of the split precisions: the
+ * planes, 30 NG (BF16X6) or 20 NG (BF16X3) bytes per transition, and 8 NG^2 per
+ * 512 transitions; up to 1 GiB of it comes from the device's default memory pool
+ * and stays there for later calls, more is given back to the device on return.
+ * (FP64: 16 NG bytes per transition and 16 NG^2 per 1,024, from the pool.)
+ * eps and w are formed in FP64, eps^-1
  * by block Gauss-Jordan elimination of eps without pivoting: eps is similar,
  * through V^1/2 where no v_G is zero, to 1 + 2 kappa V^1/2 X V^1/2, V = diag(v),
  * whose pivots are >= 1.  cuSOLVER's pivoted LU of eps takes over when a v_G is
@@ -450,7 +455,9 @@ int bse_xpy(int32_t n, int32_t k, const bse_c128* Z, const bse_c128* L, int64_t 
  *              BSE_PREC_BF16X6 / BF16X3: A and B split once into BF16 pieces
  *              and the matvecs run on the tensor cores (FP32 accumulation in
  *              K segments, FP64 results); workspace 2 x 12 N^2 bytes (BF16X6)
- *              and up to 512 MiB of partial sums.
+ *              and up to 512 MiB of partial sums.  Planes of up to 1 GiB per
+ *              matrix and the partial sums stay in the device's default memory
+ *              pool for later calls, larger planes go back to the device.
  *              The residual floor then scales with ~1e-7 of the off-diagonal
  *              part of A (A's diagonal is applied in FP64): keep tol_ev above it.
  *   E_out      [nev] device, ascending exciton energies (eV)

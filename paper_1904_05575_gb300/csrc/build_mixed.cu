@@ -1663,6 +1663,22 @@ struct DevMem {
   T* as() const { return static_cast<T*>(ptr); }
 };
 
+// Scratch of one call: from the stream-ordered pool, which keeps it for the next
+// call (cudaMalloc and cudaFree of hundreds of MB take longer than the products),
+// where the group it belongs to takes at most kPoolGroupBytes; larger groups go
+// back to the device with the object (a call syncs before it returns).
+constexpr size_t kPoolGroupBytes = 1ull << 30;
+struct Scratch {
+  std::unique_ptr<DeviceBuffer> pooled;
+  DevMem own;
+  Scratch(size_t bytes, size_t group_bytes, cudaStream_t s) {
+    if (group_bytes > kPoolGroupBytes) own = DevMem(bytes);
+    else pooled.reset(new DeviceBuffer(bytes, s));
+  }
+  template <class T>
+  T* as() const { return static_cast<T*>(pooled ? pooled->ptr : own.ptr); }
+};
+
 template <class T>
 DevMem upload_mem(const std::vector<T>& v) {
   DevMem m(v.size() * sizeof(T));
@@ -2661,10 +2677,6 @@ __global__ void __launch_bounds__(256) k_matvec_reduce(int n, int ncols, int nse
   out[o] = y;
 }
 
-// Planes up to this size (one matrix, N = 9,450) come from the stream-ordered
-// pool, which keeps them for the next call; larger ones go back to the device
-// when the object goes.
-constexpr size_t kMatvecPoolBytes = 1ull << 30;
 constexpr size_t kMatvecPartBytes = (size_t)512 << 20;   // most scratch for split-K partial sums
 }  // namespace
 
@@ -2682,9 +2694,8 @@ struct TcMatvec {
   bool has_b = false;
   const bse_c128* A = nullptr;   // caller's A (its diagonal, in FP64)
   int64_t ld = 0;
-  std::unique_ptr<DeviceBuffer> ap, bp, vp, part, err;
-  DevMem ap_large, bp_large;     // planes above kMatvecPoolBytes
-  __nv_bfloat16 *a_planes = nullptr, *b_planes = nullptr;
+  std::unique_ptr<Scratch> ap, bp;     // planes of A, B
+  std::unique_ptr<DeviceBuffer> vp, part, err;
   struct TileList {
     std::vector<tc::Tile> host;            // kept until the copy has been read
     std::unique_ptr<DeviceBuffer> dev;
@@ -2739,13 +2750,8 @@ TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t 
   m->split_cols = (int)std::max<size_t>(1, std::min<size_t>(kmax, kMatvecPartBytes / col_bytes));
   m->part.reset(new DeviceBuffer(m->split_cols * col_bytes, s));
   const size_t mat_bytes = (size_t)m->planes * n * m->Kp * 2;
-  auto planes_of = [&](std::unique_ptr<DeviceBuffer>& pooled, DevMem& large) {
-    if (mat_bytes > kMatvecPoolBytes) large = DevMem(mat_bytes);
-    else pooled.reset(new DeviceBuffer(mat_bytes, s));
-    return static_cast<__nv_bfloat16*>(large.ptr ? large.ptr : pooled->ptr);
-  };
-  m->a_planes = planes_of(m->ap, m->ap_large);
-  if (B) m->b_planes = planes_of(m->bp, m->bp_large);
+  m->ap.reset(new Scratch(mat_bytes, mat_bytes, s));
+  if (B) m->bp.reset(new Scratch(mat_bytes, mat_bytes, s));
   const size_t v_bytes = (size_t)tc::b_planes(m->pieces) * m->kmax_rows * m->Kp * 2;
   m->vp.reset(new DeviceBuffer(v_bytes, s));
   BSE_CUDA(cudaMemsetAsync(m->vp->ptr, 0, v_bytes, s));
@@ -2754,13 +2760,13 @@ TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t 
   for (int which = 0; which < (B ? 2 : 1); ++which) {
     SplitArgs sa{reinterpret_cast<const double2*>(which ? B : A), SPLIT_DENSE, nullptr, 0, 0, n,
                  m->Kp, n, m->pieces, 1, nullptr,
-                 which ? m->b_planes : m->a_planes, n, 0};
+                 (which ? m->bp : m->ap)->as<__nv_bfloat16>(), n, 0};
     sa.src_ld = ld;
     sa.zero_diag = which == 0;
     launch_split(sa, s);
   }
-  m->ma_a = make_plane_map(m->a_planes, m->Kp, n, m->planes, tc::BM);
-  if (B) m->ma_b = make_plane_map(m->b_planes, m->Kp, n, m->planes, tc::BM);
+  m->ma_a = make_plane_map(m->ap->as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
+  if (B) m->ma_b = make_plane_map(m->bp->as<__nv_bfloat16>(), m->Kp, n, m->planes, tc::BM);
   m->mb_v = make_plane_map(m->vp->as<__nv_bfloat16>(), m->Kp, m->kmax_rows,
                            tc::b_planes(m->pieces), m->nt);
   matvec_tiles(m.get(), 1, true, s);   // uploaded here: later products may be captured
@@ -2952,12 +2958,12 @@ void rpa_x_mixed(int nk, int nv, int nc, int ng, const double* e_v, const double
   const int nt = tile_cols(round_up(ng, 32), kspan);
   tc::GemmShape sh = make_shape(nt, kspan, pieces);
   sh.wait = call_wait_cycles();
-  // stream-ordered workspace: hundreds of MB of cudaMalloc and cudaFree per call
-  // took longer than the product
-  DeviceBuffer f((size_t)ntr * sizeof(double), s);
-  DeviceBuffer ap((size_t)tc::a_planes(pieces) * ng * kp * 2, s);
-  DeviceBuffer bp((size_t)tc::b_planes(pieces) * ng * kp * 2, s);
-  DeviceBuffer part((size_t)splits * ng * ng * sizeof(float2), s);
+  const size_t f_bytes = (size_t)ntr * sizeof(double),
+               a_bytes = (size_t)tc::a_planes(pieces) * ng * kp * 2,
+               b_bytes = (size_t)tc::b_planes(pieces) * ng * kp * 2,
+               part_bytes = (size_t)splits * ng * ng * sizeof(float2);
+  const size_t all = f_bytes + a_bytes + b_bytes + part_bytes;
+  Scratch f(f_bytes, all, s), ap(a_bytes, all, s), bp(b_bytes, all, s), part(part_bytes, all, s);
   DeviceBuffer err(2 * sizeof(int), s);
   BSE_CUDA(cudaMemsetAsync(err.ptr, 0, 2 * sizeof(int), s));
   {
