@@ -440,37 +440,60 @@ __global__ void k_conj(int n, TcMatvecIo io, const double2* rho, double2* y) {
 // per frequency.  The tail of the fraction is kept as num / den, so that a
 // level is two dependent FMAs (num' = (z^2 - alpha) num - beta^2 den, den' =
 // num) instead of a division (11 dependent FP64 operations of about 115 clocks
-// each); a power of two is taken out every 8 levels.
+// each).  A power of two is taken out every 8 levels; where num leaves the range
+// of FP64 within them (z^2 beyond 1e38 or below 1e-38: the tail of a recursion
+// that has ended has alpha = 0) the 8 are done again with one after each level.
+struct LzTail {
+  double nr, ni, dr, di;   // num, den
+  __device__ __forceinline__ int exponent() const {   // of the larger part of num, biased
+    return max((__double2hiint(nr) >> 20) & 0x7FF, (__double2hiint(ni) >> 20) & 0x7FF);
+  }
+  __device__ __forceinline__ void rescale() {
+    const int e = max(exponent(), 1);
+    if (e >= 0x7FE || (nr == 0.0 && ni == 0.0)) return;
+    const double sc = __longlong_as_double((long long)(2046 - e) << 52);
+    nr *= sc;
+    ni *= sc;
+    dr *= sc;
+    di *= sc;
+  }
+  // one level up: num' = (zr - alpha + i zi) num - b2 den, den' = num
+  __device__ __forceinline__ void level(double zr, double zi, double alpha, double b2) {
+    const double a = zr - alpha;
+    const double tr = fma(a, nr, fma(-zi, ni, -b2 * dr));
+    const double ti = fma(a, ni, fma(zi, nr, -b2 * di));
+    dr = nr;
+    di = ni;
+    nr = tr;
+    ni = ti;
+  }
+};
 __global__ void k_lanczos_eps(int m, const double* coef, double nv2, int n_omega,
                               const double* omega, double delta, double pref, double2* eps) {
   const int iw = blockIdx.x * blockDim.x + threadIdx.x;
   if (iw >= n_omega) return;
   const double w = omega[iw];
   const double zr = w * w - delta * delta, zi = 2.0 * w * delta;   // (w + i d)^2
-  double nr = zr - coef[2 * (m - 1)], ni = zi, dr = 1.0, di = 0.0;
-  for (int j = m - 2; j >= 0;) {
-    const int e = max((__double2hiint(nr) >> 20) & 0x7FF, (__double2hiint(ni) >> 20) & 0x7FF);
-    if (e > 0 && e < 0x7FE) {
-      const double sc = __longlong_as_double((long long)(2046 - e) << 52);
-      nr *= sc;
-      ni *= sc;
-      dr *= sc;
-      di *= sc;
-    }
+  LzTail t{zr - coef[2 * (m - 1)], zi, 1.0, 0.0};
+  for (int j0 = m - 2; j0 >= 0; j0 -= 8) {
+    t.rescale();
+    const LzTail before = t;
 #pragma unroll
-    for (int u = 0; u < 8; ++u, --j) {
-      if (j < 0) break;
-      const double a = zr - coef[2 * j], b2 = coef[2 * j + 1];
-      const double tr = fma(a, nr, fma(-zi, ni, -b2 * dr));
-      const double ti = fma(a, ni, fma(zi, nr, -b2 * di));
-      dr = nr;
-      di = ni;
-      nr = tr;
-      ni = ti;
+    for (int u = 0; u < 8; ++u)
+      if (j0 - u >= 0) t.level(zr, zi, coef[2 * (j0 - u)], coef[2 * (j0 - u) + 1]);
+    const int e = t.exponent();
+    if (e == 0 || e == 0x7FF) {
+      t = before;
+#pragma unroll 1
+      for (int j = j0; j >= 0 && j > j0 - 8; --j) {
+        t.level(zr, zi, coef[2 * j], coef[2 * j + 1]);
+        t.rescale();
+      }
     }
   }
-  const double g = pref * nv2 / fma(nr, nr, ni * ni);   // 1 / (num / den) = den conj(num) / |num|^2
-  eps[iw] = make_double2(1.0 - g * fma(dr, nr, di * ni), -g * fma(di, nr, -dr * ni));
+  t.rescale();   // |num|^2 below
+  const double g = pref * nv2 / fma(t.nr, t.nr, t.ni * t.ni);   // 1 / (num / den) = den conj(num) / |num|^2
+  eps[iw] = make_double2(1.0 - g * fma(t.dr, t.nr, t.di * t.ni), -g * fma(t.di, t.nr, -t.dr * t.ni));
 }
 
 // diff[0] = max |a - b|, diff[1] = max |b| over the grid (one block)
