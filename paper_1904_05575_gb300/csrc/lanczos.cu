@@ -426,11 +426,11 @@ __global__ void k_form_pm(int n, const double2* A, const double2* B, int64_t ld,
   }
 }
 
-// y = conj(rho), split for the first product where that runs on the tensor cores
-__global__ void k_conj(int n, TcMatvecIo io, const double2* rho, double2* y) {
+// y = scale conj(rho), split for the first product where that runs on the tensor cores
+__global__ void k_conj(int n, TcMatvecIo io, const double2* rho, double scale, double2* y) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double2 o = make_double2(rho[i].x, -rho[i].y);
+  const double2 o = make_double2(scale * rho[i].x, -scale * rho[i].y);
   y[i] = o;
   if (io.vplanes) split_into_planes(io, i, o);
 }
@@ -635,9 +635,12 @@ int spectrum_lanczos(int n, const bse_c128* A, const bse_c128* B, int64_t ld, co
   };
 
   // start: y_0 = conj(rho), v_0 = (A-B) y_0, <v_0, v_0> = y_0^H v_0
-  k_conj<<<eb, 128, 0, s>>>(n, iod, reinterpret_cast<const double2*>(rho),
-                            tc ? Yn : by0.as<double2>());
-  ++launches;
+  auto conj_rho = [&](double scale) {
+    k_conj<<<eb, 128, 0, s>>>(n, iod, reinterpret_cast<const double2*>(rho), scale,
+                              tc ? Yn : by0.as<double2>());
+    ++launches;
+  };
+  conj_rho(1.0);
   if (tc) {
     BSE_CUDA(cudaMemsetAsync(Y, 0, vb, s));   // becomes y_{-1}
     tc_matvec_products(md, s);
@@ -654,6 +657,15 @@ int spectrum_lanczos(int n, const bse_c128* A, const bse_c128* B, int64_t ld, co
     note_launches(launches);
     throw Error(nv2 == 0.0 ? BSE_ERR_ARG : BSE_ERR_NOT_PD,
                 nv2 == 0.0 ? "rho is zero" : "conj(rho)^H (A-B) conj(rho) <= 0: A-B is not positive definite");
+  }
+
+  // The FP64 steps leave x_j = beta v_j unnormalised, so alpha_0 comes from sums of
+  // the size of <v_0, v_0> alpha_0 (and of its inverse): a start vector near the
+  // ends of the FP64 range is brought to about 1 by a power of two (the fraction
+  // does not depend on it).
+  if (!tc && (nv2 < 1e-200 || nv2 > 1e200) && std::isfinite(nv2)) {
+    conj_rho(std::ldexp(1.0, -std::ilogb(nv2) / 2));
+    fp64_steps(0, 0);
   }
 
   // ten tensor-core steps as one graph

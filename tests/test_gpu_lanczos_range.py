@@ -1,6 +1,7 @@
 """eps by Lanczos at the ends of the FP64 range: a recursion that ends after one
-step (rho an eigenvector) with delta and omega towards zero, omega up to 1e60.
-A = diag(e), so eps has a closed form.  Bound 1e-10 of the largest |eps| (the
+step (rho an eigenvector) with delta and omega towards zero, omega up to 1e60;
+rho scaled by 1e-157 to 1e152 (eps - 1 is proportional to |rho|^2; subnormal
+sums to 1e-3).  A = diag(e), so eps has a closed form.  Bound 1e-10 of the largest |eps| (the
 coefficients are sums of at most 5 terms and the recursion ends exactly)."""
 import numpy as np
 import pytest
@@ -50,3 +51,15 @@ def test_large_frequencies(bse, omega):
     eps, ref = _eps(bse, rho, [omega, 2 * omega], 0.1), _closed(rho, [omega, 2 * omega], 0.1)
     assert np.isfinite(eps).all()
     assert np.abs(eps.real - ref.real).max() < 1e-10
+
+
+@pytest.mark.parametrize("scale", [1e-157, 1e-155, 1e-152, 1e-120, 1e120, 1e150, 1e152])
+def test_small_and_large_rho(bse, scale):
+    omega, one = [0.5, 2.0, 7.0], np.ones(5)
+    eps, ref = _eps(bse, scale * one, omega, 0.1), _closed(one, omega, 0.1)
+    if scale > 1.0:
+        assert np.abs((eps - 1.0) / scale / scale - (ref - 1.0)).max() < 1e-10 * np.abs(ref).max()
+    else:   # eps - 1 is lost in the real part
+        assert np.abs(eps.real - 1.0).max() < 1e-10
+        rel = 1e-3 if scale < 1e-153 else 1e-10
+        assert np.abs(eps.imag / scale / scale - ref.imag).max() < rel * np.abs(ref.imag).max()
