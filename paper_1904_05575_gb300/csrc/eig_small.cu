@@ -246,8 +246,14 @@ __global__ void __launch_bounds__(kBackThreads) k_back(int m, const double2* V, 
 }  // namespace
 
 // The k lowest eigenpairs of the real symmetric tridiagonal (d, e): bisection on
-// Sturm counts, inverse iteration.  False if a residual or an overlap is not
-// small.
+// Sturm counts, inverse iteration.  False if a residual or an overlap is larger
+// than a library eigensolve leaves them: vectors of eigenvalues kTriCluster |T|
+// apart are not orthogonalised and overlap by rounding / kTriCluster, residuals are
+// one or two units of rounding (up to 23 within groups of equal eigenvalues whose
+// shifts had to be moved apart; hundreds where such a shift met another eigenvalue,
+// which the library gets right).
+constexpr double kTriCluster = 1e-3, kTriOverlap = DBL_EPSILON / kTriCluster,
+                 kTriResidual = 32.0 * DBL_EPSILON;
 bool tridiagonal_lowest(int m, const double* d, const double* e, int k, double* lam, double* Z) {
   double lo = DBL_MAX, hi = -DBL_MAX, e2max = 0.0;
   for (int i = 0; i < m; ++i) {
@@ -293,7 +299,7 @@ bool tridiagonal_lowest(int m, const double* d, const double* e, int k, double* 
   uint64_t seed = 88172645463325252ull;
   int cluster = 0;   // first vector of the current group of close eigenvalues
   for (int c = 0; c < k; ++c) {
-    if (c > 0 && lam[c] - lam[c - 1] > 1e-3 * norm) cluster = c;
+    if (c > 0 && lam[c] - lam[c - 1] > kTriCluster * norm) cluster = c;
     double shift = lam[c];   // (equal eigenvalues: shifts a few ulp apart)
     if (c > cluster && shift - shift_prev < 10.0 * tiny) shift = shift_prev + 10.0 * tiny;
     shift_prev = shift;
@@ -363,12 +369,12 @@ bool tridiagonal_lowest(int m, const double* d, const double* e, int k, double* 
       res = std::max(res, std::fabs(t));
       z[i] = b[i];
     }
-    if (!(res < 1e-13 * norm)) return false;
+    if (!(res < kTriResidual * norm)) return false;
     for (int g = 0; g < c; ++g) {
       const double* y = Z + (size_t)g * m;
       double t = 0.0;
       for (int i = 0; i < m; ++i) t += y[i] * z[i];
-      if (!(std::fabs(t) < 1e-11)) return false;
+      if (!(std::fabs(t) < kTriOverlap)) return false;
     }
   }
   return true;
