@@ -370,8 +370,8 @@ int bse_spectrum_tensor(int32_t n, const bse_c128* Z, const bse_c128* L, int64_t
  * split into BF16 pieces, FP32 accumulation over ranges of 512 transitions);
  * the partial sums are added in FP64.  Workspace of the split precisions: the
  * planes, 30 NG (BF16X6) or 20 NG (BF16X3) bytes per transition, and 8 NG^2 per
- * 512 transitions; up to 1 GiB of it comes from the device's default memory pool
- * and stays there for later calls, more is given back to the device on return.
+ * 512 transitions, for as many transitions at a time as fit 1 GiB, from the
+ * device's default memory pool, where it stays for later calls.
  * (FP64: 16 NG bytes per transition and 16 NG^2 per 1,024, from the pool.)
  * eps and w are formed in FP64, eps^-1
  * by block Gauss-Jordan elimination of eps without pivoting: eps is similar,

@@ -1664,15 +1664,14 @@ struct DevMem {
 };
 
 // Scratch of one call: from the stream-ordered pool, which keeps it for the next
-// call (cudaMalloc and cudaFree of hundreds of MB take longer than the products),
-// where the group it belongs to takes at most kPoolGroupBytes; larger groups go
-// back to the device with the object (a call syncs before it returns).
-constexpr size_t kPoolGroupBytes = 1ull << 30;
+// call, up to kPoolBytes; a larger one goes back to the device with the object (a
+// call syncs before it returns).
+constexpr size_t kPoolBytes = 1ull << 30;
 struct Scratch {
   std::unique_ptr<DeviceBuffer> pooled;
   DevMem own;
-  Scratch(size_t bytes, size_t group_bytes, cudaStream_t s) {
-    if (group_bytes > kPoolGroupBytes) own = DevMem(bytes);
+  Scratch(size_t bytes, cudaStream_t s) {
+    if (bytes > kPoolBytes) own = DevMem(bytes);
     else pooled.reset(new DeviceBuffer(bytes, s));
   }
   template <class T>
@@ -2750,8 +2749,8 @@ TcMatvec* tc_matvec_create(int n, const bse_c128* A, const bse_c128* B, int64_t 
   m->split_cols = (int)std::max<size_t>(1, std::min<size_t>(kmax, kMatvecPartBytes / col_bytes));
   m->part.reset(new DeviceBuffer(m->split_cols * col_bytes, s));
   const size_t mat_bytes = (size_t)m->planes * n * m->Kp * 2;
-  m->ap.reset(new Scratch(mat_bytes, mat_bytes, s));
-  if (B) m->bp.reset(new Scratch(mat_bytes, mat_bytes, s));
+  m->ap.reset(new Scratch(mat_bytes, s));
+  if (B) m->bp.reset(new Scratch(mat_bytes, s));
   const size_t v_bytes = (size_t)tc::b_planes(m->pieces) * m->kmax_rows * m->Kp * 2;
   m->vp.reset(new DeviceBuffer(v_bytes, s));
   BSE_CUDA(cudaMemsetAsync(m->vp->ptr, 0, v_bytes, s));
@@ -2865,10 +2864,10 @@ __global__ void k_rpa_inv_sqrt_gap(int64_t ntr, int nv, int nc, const double* e_
   }
 }
 
-__global__ void k_rpa_reduce(const float2* part, int splits, int64_t nn, double2* x) {
+__global__ void k_rpa_reduce(const float2* part, int splits, int64_t nn, bool add, double2* x) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nn;
        i += (int64_t)gridDim.x * blockDim.x) {
-    double sx = 0.0, sy = 0.0;
+    double sx = add ? x[i].x : 0.0, sy = add ? x[i].y : 0.0;
 #pragma unroll 8
     for (int s = 0; s < splits; ++s) {
       const float2 p = part[(int64_t)s * nn + i];
@@ -2887,7 +2886,7 @@ __global__ void k_rpa_reduce(const float2* part, int splits, int64_t nn, double2
 struct RpaSplitArgs {
   const double2* m;
   const double* f;
-  int64_t ntr, kp;
+  int64_t ntr, kp;        // transitions left; columns of the planes (a multiple of 64)
   int ng;
   __nv_bfloat16 *a, *b;   // [2P][ng][kp], [3P][ng][kp]
 };
@@ -2958,30 +2957,27 @@ void rpa_x_mixed(int nk, int nv, int nc, int ng, const double* e_v, const double
   const int nt = tile_cols(round_up(ng, 32), kspan);
   tc::GemmShape sh = make_shape(nt, kspan, pieces);
   sh.wait = call_wait_cycles();
-  const size_t f_bytes = (size_t)ntr * sizeof(double),
-               a_bytes = (size_t)tc::a_planes(pieces) * ng * kp * 2,
-               b_bytes = (size_t)tc::b_planes(pieces) * ng * kp * 2,
-               part_bytes = (size_t)splits * ng * ng * sizeof(float2);
-  const size_t all = f_bytes + a_bytes + b_bytes + part_bytes;
-  Scratch f(f_bytes, all, s), ap(a_bytes, all, s), bp(b_bytes, all, s), part(part_bytes, all, s);
+  // The workspace comes from the stream-ordered pool, which keeps it for the next
+  // call (hundreds of MB of cudaMalloc and cudaFree per call took longer than the
+  // product), so the transitions go in chunks whose planes and partial sums take
+  // at most kPoolBytes.  The sums over the chunks are added in the order of one.
+  const size_t split_bytes = (size_t)(tc::a_planes(pieces) + tc::b_planes(pieces)) * ng * kspan * 2 +
+                             (size_t)ng * ng * sizeof(float2);
+  const int most = (int)std::max<size_t>(1, std::min<size_t>(splits, kPoolBytes / split_bytes));
+  const int chunks = (splits + most - 1) / most, per = (splits + chunks - 1) / chunks;
+  const int64_t kc = (int64_t)per * kspan;                // transitions per chunk
+  DeviceBuffer f((size_t)ntr * sizeof(double), s);
+  DeviceBuffer ap((size_t)tc::a_planes(pieces) * ng * kc * 2, s);
+  DeviceBuffer bp((size_t)tc::b_planes(pieces) * ng * kc * 2, s);
+  DeviceBuffer part((size_t)per * ng * ng * sizeof(float2), s);
   DeviceBuffer err(2 * sizeof(int), s);
   BSE_CUDA(cudaMemsetAsync(err.ptr, 0, 2 * sizeof(int), s));
-  {
-    Phase ph("rpa_split", s);
-    k_rpa_inv_sqrt_gap<<<(int)std::min<int64_t>((ntr + 255) / 256, 152 * 8), 256, 0, s>>>(
-        ntr, nv, nc, e_v, e_c_kq, f.as<double>());
-    const RpaSplitArgs sa{reinterpret_cast<const double2*>(m), f.as<double>(), ntr, kp, ng,
-                          ap.as<__nv_bfloat16>(), bp.as<__nv_bfloat16>()};
-    const dim3 grid((unsigned)(kp / 64), (unsigned)((ng + 31) / 32));
-    if (pieces == 3)
-      k_rpa_split<3><<<grid, 256, 0, s>>>(sa);
-    else
-      k_rpa_split<2><<<grid, 256, 0, s>>>(sa);
-    BSE_CUDA(cudaGetLastError());
-    note_launches(2);
-  }
+  k_rpa_inv_sqrt_gap<<<(int)std::min<int64_t>((ntr + 255) / 256, 152 * 8), 256, 0, s>>>(
+      ntr, nv, nc, e_v, e_c_kq, f.as<double>());
+  BSE_CUDA(cudaGetLastError());
+  note_launches(1);
   std::vector<tc::Tile> tiles;
-  for (int sp = 0; sp < splits; ++sp)
+  for (int sp = 0; sp < per; ++sp)
     for (int m0 = 0; m0 < ng; m0 += tc::BM)
       for (int n0 = 0; n0 < ng; n0 += nt)
         tiles.push_back({m0, std::min(tc::BM, ng - m0), n0, n0, std::min(nt, ng - n0), m0, sp,
@@ -2989,22 +2985,38 @@ void rpa_x_mixed(int nk, int nv, int nc, int ng, const double* e_v, const double
   DeviceBuffer dtiles(tiles.size() * sizeof(tc::Tile), s);
   BSE_CUDA(cudaMemcpyAsync(dtiles.ptr, tiles.data(), tiles.size() * sizeof(tc::Tile),
                            cudaMemcpyHostToDevice, s));
-  const CUtensorMap ma = make_plane_map(ap.as<__nv_bfloat16>(), (int)kp, ng, tc::a_planes(pieces),
+  const CUtensorMap ma = make_plane_map(ap.as<__nv_bfloat16>(), (int)kc, ng, tc::a_planes(pieces),
                                         tc::BM);
-  const CUtensorMap mb = make_plane_map(bp.as<__nv_bfloat16>(), (int)kp, ng, tc::b_planes(pieces),
+  const CUtensorMap mb = make_plane_map(bp.as<__nv_bfloat16>(), (int)kc, ng, tc::b_planes(pieces),
                                         nt);
-  {
-    Phase ph("rpa_x_gemm", s);
-    launch_gemm(ma, mb, dtiles.as<tc::Tile>(), (int)tiles.size(), sh, RpaPartialEpi{part.as<float2>(), ng},
-                err.as<int>(), s);
-  }
-  {
-    Phase ph("rpa_reduce", s);
-    const int64_t nn = (int64_t)ng * ng;
-    k_rpa_reduce<<<(int)std::min<int64_t>((nn + 255) / 256, 152 * 8), 256, 0, s>>>(
-        part.as<float2>(), splits, nn, x_out);
-    BSE_CUDA(cudaGetLastError());
-    note_launches(1);
+  for (int sp0 = 0; sp0 < splits; sp0 += per) {
+    const int ns = std::min(per, splits - sp0);
+    const int64_t k0 = (int64_t)sp0 * kspan;
+    {
+      Phase ph("rpa_split", s);
+      const RpaSplitArgs sa{reinterpret_cast<const double2*>(m) + k0 * ng, f.as<double>() + k0, ntr - k0,
+                            kc, ng, ap.as<__nv_bfloat16>(), bp.as<__nv_bfloat16>()};
+      const dim3 grid((unsigned)(ns * kspan / 64), (unsigned)((ng + 31) / 32));
+      if (pieces == 3)
+        k_rpa_split<3><<<grid, 256, 0, s>>>(sa);
+      else
+        k_rpa_split<2><<<grid, 256, 0, s>>>(sa);
+      BSE_CUDA(cudaGetLastError());
+      note_launches(1);
+    }
+    {
+      Phase ph("rpa_x_gemm", s);
+      launch_gemm(ma, mb, dtiles.as<tc::Tile>(), (int)(tiles.size() / per * ns), sh,
+                  RpaPartialEpi{part.as<float2>(), ng}, err.as<int>(), s);
+    }
+    {
+      Phase ph("rpa_reduce", s);
+      const int64_t nn = (int64_t)ng * ng;
+      k_rpa_reduce<<<(int)std::min<int64_t>((nn + 255) / 256, 152 * 8), 256, 0, s>>>(
+          part.as<float2>(), ns, nn, sp0 > 0, x_out);
+      BSE_CUDA(cudaGetLastError());
+      note_launches(1);
+    }
   }
   int herr = 0;
   BSE_CUDA(cudaMemcpyAsync(&herr, err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));

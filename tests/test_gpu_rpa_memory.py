@@ -1,7 +1,8 @@
 """Device memory that stays in use after a split-precision screening: at most the
-1 GiB that the pool may keep, whatever the number of transitions; a workspace
-above that is given back on return.  64 MiB allowance for the pool's block size
-and the library's small buffers."""
+1 GiB of workspace that the pool may keep, whatever the number of transitions
+(they go in chunks), and 8 bytes per transition.  64 MiB allowance for the pool's
+block size and the library's small buffers.  The result of several chunks, the
+last one shorter, against numpy (BF16x6: 1e-6 of the largest |w|)."""
 import numpy as np
 import pytest
 
@@ -33,27 +34,22 @@ def test_workspace_after_the_call(bse):
 
     w = torch.empty((ng, ng), dtype=torch.complex128, device="cuda")
     call = lambda a: bse.bse_rpa_screening(*a, 250.0, w, precision=2)  # noqa: E731
-    # 16,000, 160,000 and 400,000 transitions: planes of 0.1, 0.96 and 2.4 GB,
-    # partial sums of 0.01, 0.1 and 0.25 GB
+    # 16,000 and 160,000 transitions (0.1 and 0.99 GiB), 400,000 and 451,000 (2.5 and
+    # 2.8 GiB of workspace at once)
     small, below, above = inputs(40, 20, 20), inputs(400, 20, 20), inputs(1000, 20, 20)
+    ragged = inputs(1000, 11, 41)
     torch.cuda.empty_cache()
     call(small)      # library handles, module load
-    used = [torch.cuda.mem_get_info()[0]]
-    for a in (above, below, above):
+    free = [torch.cuda.mem_get_info()[0]]
+    for a in (below, above, ragged):
         call(a)
         torch.cuda.synchronize()
-        used.append(torch.cuda.mem_get_info()[0])
-    free0, after_above, after_below, after_all = used
-    assert free0 - after_above <= SLACK            # given back
-    assert free0 - after_below <= GIB + SLACK      # kept for the next call, bounded
-    assert after_below - after_all <= SLACK        # and not added to
-    # the pool's memory and the device's give the same result
-    w1 = w.clone()
-    call(above)
-    assert torch.equal(w, w1)
-    e_v, e_c, m, v = (x.cpu().numpy() for x in below)
-    call(below)
-    t = (m / np.sqrt(e_c[:, None, :] - e_v[:, :, None])[..., None]).reshape(-1, ng)
-    eps = np.eye(ng) + 2.0 * 27.211386245988 / (400 * 250.0) * (t.conj().T @ t) * v[None, :]
-    ref = v[:, None] * np.linalg.inv(eps)
-    assert np.abs(w.cpu().numpy() - ref).max() < 1e-6 * np.abs(ref).max()
+        free.append(torch.cuda.mem_get_info()[0])
+    assert free[0] - min(free) <= GIB + SLACK
+    for a in (above, ragged):
+        call(a)
+        e_v, e_c, m, v = (x.cpu().numpy() for x in a)
+        t = (m / np.sqrt(e_c[:, None, :] - e_v[:, :, None])[..., None]).reshape(-1, ng)
+        eps = np.eye(ng) + 2.0 * 27.211386245988 / (len(e_v) * 250.0) * (t.conj().T @ t) * v[None, :]
+        ref = v[:, None] * np.linalg.inv(eps)
+        assert np.abs(w.cpu().numpy() - ref).max() < 1e-6 * np.abs(ref).max()
