@@ -105,7 +105,7 @@ namespace bse {
 // (and what rounds there) an infinity.  The word shifted left by 3 holds the
 // low 9 exponent bits above the 23 fraction bits, so re-biasing (896 = 384 mod
 // 512) and rounding are one three-operand add.
-__host__ __device__ __forceinline__ uint32_t f64w_to_f32_bits(uint32_t lo, uint32_t hi) {
+__device__ __forceinline__ uint32_t f64w_to_f32_bits(uint32_t lo, uint32_t hi) {
   const uint32_t f = ((hi << 3) | (lo >> 29)) - (384u << 23) + ((lo >> 28) & 1u);
   const uint32_t mag = hi & 0x7FFFFFFFu;
   const bool in = mag - (897u << 20) < (254u << 20);   // biased FP32 exponent in [1, 254]
@@ -114,14 +114,14 @@ __host__ __device__ __forceinline__ uint32_t f64w_to_f32_bits(uint32_t lo, uint3
 }
 
 // The same where |x| lies in [2^-126, 2^128), without the range check: the
-// caller checks `out` (the largest f64w_range of a group of words) once and
-// converts the group again with the function above if it is not below
-// kF64InRange (zeros and padding).
+// caller checks the largest f64w_range of a group of words once and converts the
+// group again with the function above if it is not below kF64InRange (zeros and
+// padding).
 constexpr uint32_t kF64InRange = 254u << 20;
-__host__ __device__ __forceinline__ uint32_t f64w_range(uint32_t hi) {
+__device__ __forceinline__ uint32_t f64w_range(uint32_t hi) {
   return (hi & 0x7FFFFFFFu) - (897u << 20);
 }
-__host__ __device__ __forceinline__ uint32_t f64w_to_f32_in_range(uint32_t lo, uint32_t hi) {
+__device__ __forceinline__ uint32_t f64w_to_f32_in_range(uint32_t lo, uint32_t hi) {
   return (hi & 0x80000000u) | (((hi << 3) | (lo >> 29)) - (384u << 23) + ((lo >> 28) & 1u));
 }
 

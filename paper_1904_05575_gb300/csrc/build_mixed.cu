@@ -1364,8 +1364,11 @@ Stage2Form stage2_form(const Stage2Args& a, int npair) {
   if (stage2_multi_pairs(a) >= 2) return S2F_MULTI;
   if (a.rows_x <= 16 && a.rows_t <= 16) return S2F_PIPE;
   // nearly square blocks that one tile of 2 x 3 or 2 x 5 outputs per thread
-  // covers: 24 x 24 (with 15 x 15 and 4 x 4: 1,231 us against 1,465 us for
-  // k_stage2_rows), 40 x 40 (755 against 974 us)
+  // covers: against k_stage2_rows at 4,096 pairs and NG = 181, 21 x 21 192 / 217
+  // us, 24 x 24 192 / 244, 33 x 33 486 / 571, 36 x 36 486 / 573, 40 x 40 487 / 652
+  // (25 x 25 474 / 451; 27 x 27 to 32 x 32, where 40 x 40 computes 1.6 to 2.2 times
+  // the outputs, 477 / 343: the tile is kept for its start with few pairs, 104 / 95
+  // at 729)
   int64_t outputs = 0;
   const Stage2Form tiles = stage2_tile_form(a, &outputs);
   if (tiles == S2F_24 || tiles == S2F_40) return tiles;

@@ -17,8 +17,8 @@
 // back on the library where it fails or m is too large.  Bound by the latency
 // of the reduction's chain per column (two grid exchanges, a square root, two
 // divisions and three block sums, about 7 us): the projected problems of that
-// solve take 2.6 instead of 6.4 ms per iteration, the solve 97 instead of 166
-// (72.5 with the tall-skinny products of davidson.cu).
+// solve take 2.6 instead of 6.4 ms per iteration, the solve 95 to 97 instead of
+// 166 (72.5 with the tall-skinny products of davidson.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -121,7 +121,9 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_hetrd(TrdArgs a) {
     double2 *col = a.col + (int64_t)(j & 1) * m, *next = a.col + (int64_t)((j + 1) & 1) * m;
     double2* p = a.p + (int64_t)(j & 1) * m;
     if (!trd_barrier(a, arrived += nb, &ok_s)) return;
-    // the reflector of column j (every block: the same bits)
+    // the reflector of column j (every block: the same bits); a column whose
+    // squares fall out of the range of FP64 (below 1e-154) gives an infinite scale,
+    // T is not finite and the library serves the matrix
     double s2 = 0.0;
     for (int i = j + 1 + tid; i < m; i += kTrdThreads) {
       const double2 x = __ldcg(col + i);

@@ -543,7 +543,10 @@ __global__ void k_rpa_w(int ng, const double* v, const double2* inv, double2* w)
 // kGjNb x kGjNb pivot block and updates its own columns.  Bound by the FP64
 // pipe: 4 NG^3 FMAs (0.9 ms at NG = 500 and 1.8 FMAs per clock and SM), and the
 // serial pivot blocks; 1.7 ms at NG = 500, where the pivoted LU and solve of the
-// library took about 6 ms.
+// library took about 6 ms.  Whole FP64 calls of 128 transitions with the library's
+// LU and with this, the rest being small: NG = 59 1.05 and 0.25 ms, 400 6.5 and
+// 1.5, 700 14.3 and 5.4, 1,000 26.2 and 10.6, 1,216 (the last with 160 KB of
+// columns per block) 37.5 and 14.9.
 constexpr int kGjNb = 16, kGjThreads = 256, kGjMaxSmem = 160 * 1024;
 
 struct GjArgs {
