@@ -540,7 +540,11 @@ __global__ void k_rpa_w(int ng, const double* v, const double2* inv, double2* w)
 // Each block owns a few columns and keeps them in shared memory from load to
 // result; a step eliminates kGjNb columns: the blocks that own them publish
 // them (double-buffered, one grid barrier per step), every block inverts the
-// kGjNb x kGjNb pivot block and updates its own columns.  Bound by the FP64
+// kGjNb x kGjNb pivot block and updates its own columns.  The diagonal elements
+// are the only ones that are not small: a step's products are summed by themselves
+// before they go into one, or its n updates would leave sqrt(n) roundings in it
+// (w of NG = 150 and 300 off by 1.0e-15, by 5.4 and 6.7e-16 with LU and solve, by
+// 3.6 and 5.1e-16 so).  Bound by the FP64
 // pipe: 4 NG^3 FMAs (0.9 ms at NG = 500 and 1.8 FMAs per clock and SM), and the
 // serial pivot blocks; 1.7 ms at NG = 500, where the pivoted LU and solve of the
 // library took about 6 ms.  Whole FP64 calls of 128 transitions with the library's
@@ -586,7 +590,7 @@ __device__ __forceinline__ bool gj_barrier(const GjArgs& a, int target, int* ok_
 
 __global__ void __launch_bounds__(kGjThreads, 1) k_gj_screening(GjArgs a) {
   extern __shared__ double2 gj_cols[];            // [cols][n]
-  __shared__ double2 D[kGjNb][kGjNb + 1], R[kGjNb][8], rp_s;
+  __shared__ double2 D[kGjNb][kGjNb + 1], R[kGjNb][8], diag[8], rp_s;
   __shared__ int ok_s;
   const int n = a.n, c0 = blockIdx.x * a.cols, nc = min(a.cols, n - c0);
   const int tid = threadIdx.x, dr = tid / kGjNb, dc = tid % kGjNb;
@@ -654,6 +658,11 @@ __global__ void __launch_bounds__(kGjThreads, 1) k_gj_screening(GjArgs a) {
           }
         }
         R[m][c] = o;
+      } else if (tid < kGjNb * 8 + cn) {   // the products of a diagonal element by themselves
+        const int c = tid - kGjNb * 8, j = c0 + cb + c;
+        double2* x = gj_cols + (cb + c) * n + j;
+        diag[c] = *x;
+        *x = make_double2(0.0, 0.0);
       }
       __syncthreads();
       for (int c4 = 0; c4 < cn; c4 += 4) {
@@ -684,6 +693,11 @@ __global__ void __launch_bounds__(kGjThreads, 1) k_gj_screening(GjArgs a) {
           for (int c = 0; c < 4; ++c)
             if (c4 + c < cn) gj_cols[(cb + c4 + c) * n + r] = x[c];
         }
+      }
+      const int cd = (tid - c0 - cb) & (kGjThreads - 1), r = c0 + cb + cd;   // (r is this thread's row)
+      if (cd < cn && !(r >= k0 && r < k0 + nb)) {
+        double2* x = gj_cols + (cb + cd) * n + r;
+        *x = make_double2(diag[cd].x + x->x, diag[cd].y + x->y);
       }
       __syncthreads();
     }
