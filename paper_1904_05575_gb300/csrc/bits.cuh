@@ -113,18 +113,6 @@ __device__ __forceinline__ uint32_t f64w_to_f32_bits(uint32_t lo, uint32_t hi) {
   return (hi & 0x80000000u) | r;
 }
 
-// The same where |x| lies in [2^-126, 2^128), without the range check: the
-// caller checks the largest f64w_range of a group of words once and converts the
-// group again with the function above if it is not below kF64InRange (zeros and
-// padding).
-constexpr uint32_t kF64InRange = 254u << 20;
-__device__ __forceinline__ uint32_t f64w_range(uint32_t hi) {
-  return (hi & 0x7FFFFFFFu) - (897u << 20);
-}
-__device__ __forceinline__ uint32_t f64w_to_f32_in_range(uint32_t lo, uint32_t hi) {
-  return (hi & 0x80000000u) | (((hi << 3) | (lo >> 29)) - (384u << 23) + ((lo >> 28) & 1u));
-}
-
 // FP32 -> BF16 bit pattern, round to nearest even (finite inputs).
 __device__ __forceinline__ uint32_t f32_to_bf16_rn_bits(uint32_t u) {
   return (u + 0x7FFFu + ((u >> 16) & 1u)) >> 16;

@@ -764,8 +764,11 @@ __global__ void __launch_bounds__(256) k_stage2_pipe(Stage2Args a) {
 // Bound by latency and issue together (0.4 instructions per clock and
 // scheduler with ten warps per SM at 168 registers; the packed FMA pipe 44 %
 // busy).  4 x 12 bands, NG = 181, 4,096 pairs: W^rr (144 X rows, 16 T rows)
-// 1,453 -> 863 us, W^ra (48 x 48) 1,178 -> 735 us against 32 x 32 tiles with
-// 2 x 2 outputs per thread.  stage2_rows_pays says where it is used.  Tried and slower: 4 x 4 packed outputs per thread
+// 1,453 -> 813 us, W^ra (48 x 48) 1,178 -> 718 us against 32 x 32 tiles with
+// 2 x 2 outputs per thread, whatever the values (with a faster conversion behind
+// one range check per chunk 863 and 735 us, but 1,099 and 985 where X has zeros,
+// as real matrix elements have throughout).  stage2_rows_pays says where it is
+// used.  Tried and slower than that: 4 x 4 packed outputs per thread
 // with X converted through shared memory (861 / 803 us), fewer T rows per
 // thread for more warps (8: 1,159 / 1,043 us), 20 T rows for 40 x 40 blocks.
 constexpr int S2_GC = 8, S2_RING = 4, S2_MAXTH = 160, S2_MAXPB = 8;
@@ -908,28 +911,14 @@ k_stage2_rows(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ 
     uint64_t ax[P], ay[P];
 #pragma unroll
     for (int j = 0; j < P; ++j) ax[j] = ay[j] = 0ull;
-    // the chunk's X elements, with one range check for all eight (a branch per
-    // element kept the conversions from overlapping the FMAs)
-    uint32_t xre[S2_GC], xim[S2_GC], range = 0u;
+    // the chunk's X elements, zeros (real matrix elements, padding) like any other:
+    // no branch, so the conversions overlap the FMAs
+    uint32_t xre[S2_GC], xim[S2_GC];
 #pragma unroll
     for (int g = 0; g < S2_GC; ++g) {
       const uint4 d = *reinterpret_cast<const uint4*>(xs + (xoff ^ (g * 16)));
-      range = max(range, max(f64w_range(d.y), f64w_range(d.w)));
-      xre[g] = f64w_to_f32_in_range(d.x, d.y);
-      xim[g] = f64w_to_f32_in_range(d.z, d.w) ^ xflip;
-    }
-    if (range >= kF64InRange) {
-#pragma unroll 1
-      for (int g = 0; g < S2_GC; ++g) {
-        const uint4 d = *reinterpret_cast<const uint4*>(xs + (xoff ^ (g * 16)));
-        const uint32_t re = f64w_to_f32_bits(d.x, d.y), im = f64w_to_f32_bits(d.z, d.w) ^ xflip;
-#pragma unroll
-        for (int u = 0; u < S2_GC; ++u)
-          if (u == g) {
-            xre[u] = re;
-            xim[u] = im;
-          }
-      }
+      xre[g] = f64w_to_f32_bits(d.x, d.y);
+      xim[g] = f64w_to_f32_bits(d.z, d.w) ^ xflip;
     }
 #pragma unroll
     for (int g = 0; g < S2_GC; ++g) {
@@ -1332,22 +1321,22 @@ Stage2Form stage2_tile_form(const Stage2Args& a, int64_t* outputs) {   // + outp
 }
 // The one-row form against the tiles: a tile form takes 0.37 ns per 1,000
 // outputs and plane wave once its blocks fill the GPU, the one-row form about
-// 1.15 times that, but it starts 18 us later at NG = 181 (28 against 10 us: two
-// to six warps per block, one ring of copies behind the other; 11 us at 91).  So
-// it takes the term where it computes a quarter fewer outputs and what it saves
-// on all pairs, saved = tile outputs - 1.15 row outputs, is worth that start:
-// 270,000 outputs by the figures, 500,000 here, so that no measured size loses.
-// NG = 181, us, tiles / one row: 48 x 48 with 108, 216, 729 and 4,096 pairs
-// (saved 1,446) 41 / 51, 72 / 65, 217 / 155, 1,143 / 735; 144 x 16 with 64, 216,
-// 4,096 (2,176) 39 / 67, 90 / 74, 1,407 / 863; 400 x 9 with 64, 108, 4,096
-// (6,688) 70 / 88, 111 / 82, 3,640 / 1,807; 25 x 9 with 729, 2,048, 15,625 (159)
-// 41 / 55, 96 / 96, 624 / 518.  Not a quarter fewer: 25 x 16 at 4,096 pairs
-// 174 / 264, 36 x 16 229 / 252.  Against several 32 x 32 tiles the one-row form
-// is also the faster one with as many outputs where plane waves and pairs are
+// 1.1 times that, but it starts 17 us later at NG = 181 (two to six warps per
+// block, one ring of copies behind the other; 10 us at 91).  So it takes the term
+// where it computes a quarter fewer outputs and what it saves on all pairs, saved =
+// tile outputs - 1.15 row outputs, is worth that start: 340,000 outputs, with
+// which it lost at one of 190 measured points (400 x 16, 108 pairs, NG = 91, 7 %).
+// NG = 181, us, tiles / one row: 48 x 48 with 108, 216, 351, 729 and 4,096 pairs
+// (saved 1,446) 41 / 49, 72 / 63, 113 / 91, 217 / 153, 1,145 / 719; 144 x 16 with
+// 64, 108, 216, 4,096 (2,176) 39 / 49, 50 / 52, 91 / 71, 1,409 / 813; 400 x 9 with
+// 16, 64, 4,096 (6,688) 28 / 45, 70 / 61, 3,641 / 1,766; 25 x 9 with 729, 2,048,
+// 4,096 (159) 41 / 44, 96 / 100, 174 / 149.  Not a quarter fewer: 25 x 16 at 4,096
+// pairs 174 / 246, 36 x 16 231 / 235.  Against several 32 x 32 tiles the one-row
+// form is also the faster one with as many outputs where plane waves and pairs are
 // many, by a few per cent: 4,096 pairs at NG = 181, both terms of 5 x 10 bands
-// (100 x 25, 50 x 50) 2,314 / 2,193, of 7 x 7 2,314 / 2,304; at NG = 91 1,243 /
-// 1,279 and 1,243 / 1,389, with 1,024 pairs 592 / 579 and 594 / 610.
-constexpr int64_t kS2RowsSaved = 500000;
+// (100 x 25, 50 x 50) 2,314 / 2,111, of 7 x 7 2,316 / 2,234; at NG = 91 1,246 /
+// 1,217 and 1,244 / 1,341, with 1,024 pairs 592 / 561 and 595 / 592.
+constexpr int64_t kS2RowsSaved = 340000;
 constexpr int kS2RowsManyNg = 160, kS2RowsManyPairs = 2000;
 bool stage2_rows_pays(const Stage2Args& a, int npair, int64_t tile_outputs) {
   const S2Tile t = stage2_tile(a, npair);
