@@ -702,15 +702,22 @@ __global__ void __launch_bounds__(kGjThreads, 1) k_gj_screening(GjArgs a) {
       __syncthreads();
     }
   }
+  // w is written once every block knows that all of it is good: a matrix that the
+  // LU refuses too leaves w as it was
   for (int i = tid; i < n * nc; i += kGjThreads) {
     const int r = i / nc, c = i - r * nc;
     const double2 x = gj_cols[c * n + r];
     const double vg = a.v[r];
     const double2 o = make_double2(vg * x.x, vg * x.y);
     if (!isfinite(o.x) || !isfinite(o.y)) bad = true;
-    a.w[(int64_t)r * n + c0 + c] = o;
+    gj_cols[c * n + r] = o;
   }
   if (bad) atomicOr(a.bad, 1);
+  if (!gj_barrier(a, arrived += gridDim.x, &ok_s) || __ldcg(a.bad)) return;
+  for (int i = tid; i < n * nc; i += kGjThreads) {
+    const int r = i / nc, c = i - r * nc;
+    a.w[(int64_t)r * n + c0 + c] = gj_cols[c * n + r];
+  }
 }
 
 // w by the launch above; false: the matrix is left to the pivoted LU (too large
