@@ -62,11 +62,11 @@ KERNEL_SOURCES = ("paper_1904_05575_gb300/csrc/build_mixed.cu", "paper_1904_0557
                   "paper_1904_05575_gb300/csrc/bse_internal.h")
 TRAFFIC = {
     # workload: {phase: (bytes per build, sources digest at capture)}
-    "c5": {"mixed_stage2_tc": (49495153664, "6a5cd02d7839c2d6"),
-           "mixed_stage1_gemm": (25860002560, "6a5cd02d7839c2d6"),
-           "mixed_split": (50944937984, "6a5cd02d7839c2d6"),
-           "mixed_exchange": (13864601344, "6a5cd02d7839c2d6"),
-           "hermitian_complete": (20564511488, "6a5cd02d7839c2d6")},
+    "c5": {"mixed_stage2_tc": (49494622464, "95f55e3bbe54b0c2"),
+           "mixed_stage1_gemm": (25963332352, "95f55e3bbe54b0c2"),
+           "mixed_split": (50945645824, "95f55e3bbe54b0c2"),
+           "mixed_exchange": (13867299328, "95f55e3bbe54b0c2"),
+           "hermitian_complete": (20564517120, "95f55e3bbe54b0c2")},
 }
 
 
